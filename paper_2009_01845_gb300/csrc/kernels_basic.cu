@@ -19,6 +19,7 @@
 #include "device.cuh"
 #include "internal.h"
 #include "prof.h"
+#include "xfield.h"
 
 namespace qsim {
 
@@ -770,10 +771,32 @@ qs_status k_expectation(qs_state *s, const qs_pauli_term *terms, size_t count, d
         }
         groups[gi].push_back(t);
     }
+    // single X terms (a transverse field): several per read of the state
+    double field[64] = {0.0};
+    int field_terms = 0;
+    auto in_field = [&](size_t gi) {
+        if (__builtin_popcountll(masks[gi]) != 1) return false;
+        for (size_t t : groups[gi])
+            if (terms[t].z_mask) return false;
+        return true;
+    };
+    for (size_t gi = 0; gi < masks.size(); ++gi) {
+        if (!in_field(gi)) continue;
+        double c = 0.0;
+        for (size_t t : groups[gi]) c += terms[t].coeff;
+        field[__builtin_ctzll(masks[gi])] = c;
+        field_terms += c != 0.0;
+    }
+    const bool fused_field = xfield_fits(n, field_terms);
     bool first = true;
     ProfScope _ps(s->stream, KC_REDUCE);
     dim3 grid(P, s->batch);
+    if (fused_field) {
+        QS_TRY(k_xfield(s->data, n, s->ms, s->batch, s->dtype, field, s->scratch, P, false, s->stream));
+        first = false;
+    }
     for (size_t gi = 0; gi < masks.size(); ++gi) {
+        if (fused_field && in_field(gi)) continue;
         const auto &idx = groups[gi];
         for (size_t c0 = 0; c0 < idx.size(); c0 += kMaxTermsPerLaunch) {
             ExpP<double> p;
@@ -1179,11 +1202,32 @@ static qs_status expectation_noalloc_t(const V<R> *psi, int n, int batch, const 
     const dim3 grid(P, batch);
     bool first = true;
     ExpP<R> p;  // on the host stack: passed by value as kernel parameters
+    // single X terms (a transverse field): several per read of the state. A bit
+    // whose X also appears with Z bits stays with its group
+    double field[64] = {0.0};
+    uint64_t mixed = 0;
+    for (size_t t = 0; t < count; ++t) {
+        if (__builtin_popcountll(terms[t].x_mask) != 1) continue;
+        const uint64_t b = qbit(n, __builtin_ctzll(terms[t].x_mask));
+        if (terms[t].z_mask) mixed |= b;
+        field[__builtin_ctzll(b)] += terms[t].coeff;
+    }
+    int field_terms = 0;
+    for (int b = 0; b < n; ++b) {
+        if ((mixed >> b) & 1ull) field[b] = 0.0;
+        field_terms += field[b] != 0.0;
+    }
+    const bool fused_field = xfield_fits(n, field_terms);
+    if (fused_field) {
+        QS_TRY(k_xfield(psi, n, n, batch, sizeof(R) == 4 ? QS_C64 : QS_C128, field, part, P, false, stream));
+        first = false;
+    }
     for (size_t lead = 0; lead < count; ++lead) {
         // one group per distinct X mask, handled at its first occurrence
         uint64_t xb = 0;
         for (int q = 0; q < n; ++q)
             if ((terms[lead].x_mask >> q) & 1ull) xb |= qbit(n, q);
+        if (fused_field && __builtin_popcountll(xb) == 1 && !(xb & mixed)) continue;
         bool seen = false;
         for (size_t e = 0; e < lead && !seen; ++e) {
             uint64_t xe = 0;
