@@ -24,6 +24,7 @@
 #include <vector>
 
 #include "adjoint.h"
+#include "hpsi.h"
 #include "internal.h"
 #include "plan.h"
 
@@ -78,19 +79,26 @@ qs_status run_evolve(qs_state *s, const qs_pauli_term *h0, size_t n0, const qs_p
     const size_t bytes = total * amp_bytes_of(s->dtype);
     Work w{s->stream, {}};
     const double eps = s->dtype == QS_C64 ? 6e-8 : 1.2e-16;  // unit roundoff of the state's precision
-    auto applyH = [&](const std::vector<qs_pauli_term> &t, void *src, void *dst) {
-        return k_pauli_apply(view(s, src), view(s, dst), t.data(), t.size(), s->stream);
+    auto prepare = [&](double sv, HpsiOp *op, double *nu = nullptr) {
+        const std::vector<qs_pauli_term> H = mix(h0, n0, h1, n1, sv);
+        if (nu) *nu = norm_bound(H);
+        return hpsi_prepare(view(s, s->data), H.data(), H.size(), op);
+    };
+    // out = base + c H src (no base: c H src) for one or two results
+    auto applyH = [&](const HpsiOp &op, void *src, const HpsiOut &a, const HpsiOut &b, void *spare) {
+        return hpsi_apply(op, view(s, src), a, b, spare, s->stream);
     };
     auto comb = [&](void *out, std::vector<const void *> in, std::vector<cd> c) {
         return k_combine(s->dtype, out, in, c, total, s->stream);
     };
     const cd mi(0.0, -1.0);
+    HpsiOp op;
     if (solver == QS_SOLVER_EXP) {
         QS_TRY(w.alloc(bytes, 2));
-        void *term = w.bufs[0], *tmp = w.bufs[1];
+        void *term = w.bufs[0], *next = w.bufs[1];
         for (int k = 0; k < steps; ++k) {
-            const std::vector<qs_pauli_term> H = mix(h0, n0, h1, n1, (k + 0.5) * dt / T);
-            const double nu = norm_bound(H);
+            double nu;
+            QS_TRY(prepare((k + 0.5) * dt / T, &op, &nu));
             const int m = std::max(1, (int)std::ceil(nu * dt));
             const double tau = dt / m;
             // order: the first K with (nu tau)^(K+1) / (K+1)! <= eps
@@ -101,11 +109,12 @@ qs_status run_evolve(qs_state *s, const qs_pauli_term *h0, size_t n0, const qs_p
                 if (b <= eps) break;
             }
             for (int piece = 0; piece < m; ++piece) {
+                // the next Taylor term and its sum leave the application of H together
                 QS_TRY(comb(term, {s->data}, {1.0}));
                 for (int j = 1; j <= K; ++j) {
-                    QS_TRY(applyH(H, term, tmp));
-                    QS_TRY(comb(term, {tmp}, {mi * (tau / j)}));
-                    QS_TRY(comb(s->data, {s->data, term}, {1.0, 1.0}));
+                    const cd c = mi * (tau / j);
+                    QS_TRY(applyH(op, term, {next, nullptr, c}, {s->data, s->data, c}, next));
+                    std::swap(term, next);
                 }
             }
         }
@@ -113,22 +122,19 @@ qs_status run_evolve(qs_state *s, const qs_pauli_term *h0, size_t n0, const qs_p
     }
     if (solver == QS_SOLVER_RK4) {
         QS_TRY(w.alloc(bytes, 3));
-        void *acc = w.bufs[0], *yt = w.bufs[1], *hk = w.bufs[2];
+        void *acc = w.bufs[0], *ya = w.bufs[1], *yb = w.bufs[2];
         void *y = s->data;
         for (int k = 0; k < steps; ++k) {
             const double t = k * dt;
-            // stage i: hk = H(t_i) y_i, k_i = -i hk; acc gathers y + dt sum b_i k_i
-            QS_TRY(applyH(mix(h0, n0, h1, n1, t / T), y, hk));
-            QS_TRY(comb(acc, {y, hk}, {1.0, mi * (dt / 6)}));
-            QS_TRY(comb(yt, {y, hk}, {1.0, mi * (dt / 2)}));
-            QS_TRY(applyH(mix(h0, n0, h1, n1, (t + dt / 2) / T), yt, hk));
-            QS_TRY(comb(acc, {acc, hk}, {1.0, mi * (dt / 3)}));
-            QS_TRY(comb(yt, {y, hk}, {1.0, mi * (dt / 2)}));
-            QS_TRY(applyH(mix(h0, n0, h1, n1, (t + dt / 2) / T), yt, hk));
-            QS_TRY(comb(acc, {acc, hk}, {1.0, mi * (dt / 3)}));
-            QS_TRY(comb(yt, {y, hk}, {1.0, mi * dt}));
-            QS_TRY(applyH(mix(h0, n0, h1, n1, (t + dt) / T), yt, hk));
-            QS_TRY(comb(y, {acc, hk}, {1.0, mi * (dt / 6)}));
+            // stage i: k_i = -i H(t_i) y_i; acc gathers y + dt sum b_i k_i, the
+            // next stage's state goes to the buffer that does not hold y_i
+            QS_TRY(prepare(t / T, &op));
+            QS_TRY(applyH(op, y, {acc, y, mi * (dt / 6)}, {ya, y, mi * (dt / 2)}, ya));
+            QS_TRY(prepare((t + dt / 2) / T, &op));
+            QS_TRY(applyH(op, ya, {acc, acc, mi * (dt / 3)}, {yb, y, mi * (dt / 2)}, yb));
+            QS_TRY(applyH(op, yb, {acc, acc, mi * (dt / 3)}, {ya, y, mi * dt}, ya));
+            QS_TRY(prepare((t + dt) / T, &op));
+            QS_TRY(applyH(op, ya, {y, acc, mi * (dt / 6)}, {}, yb));
         }
         return QS_OK;
     }
@@ -159,7 +165,8 @@ qs_status run_evolve(qs_state *s, const qs_pauli_term *h0, size_t n0, const qs_p
                 QS_TRY(comb(yt, in, c));
                 src = yt;
             }
-            QS_TRY(applyH(mix(h0, n0, h1, n1, (t + C[i] * dt) / T), const_cast<void *>(src), w.bufs[i]));
+            QS_TRY(prepare((t + C[i] * dt) / T, &op));
+            QS_TRY(applyH(op, const_cast<void *>(src), {w.bufs[i], nullptr, 1.0}, {}, w.bufs[i]));
         }
         std::vector<const void *> in = {y};
         std::vector<cd> c = {1.0};
