@@ -21,6 +21,7 @@
 #include "adjoint.h"
 #include "plan.h"
 #include "prof.h"
+#include "small.h"
 #include "tiled.h"
 
 namespace qsim {
@@ -163,7 +164,7 @@ qs_status energy_gradient(qs_state *w, const std::vector<LGate> &G, const double
         }
     }
     const int k = tile_bits(w->dtype);
-    const bool small = n + 1 < k;  // below one tile: unfused sweep
+    const bool small = n + 1 < k;  // below one tile: the small-state kernel
     const uint64_t total_tiles = small ? (uint64_t)B : (uint64_t)B << (n + 1 - k);
     double *gpart = nullptr;
     const size_t nslot = slot_param.size();
@@ -176,15 +177,7 @@ qs_status energy_gradient(qs_state *w, const std::vector<LGate> &G, const double
     }
     for (int c = nseg - 1; c >= 0 && st == QS_OK; --c) {
         if (small) {
-            for (const LGate &g : rev[c]) {
-                if (g.kind == kKindGrad)
-                    st = k_grad_small(w, g, gpart + (size_t)g.grad_slot * total_tiles);
-                else if (g.param_index >= 0)
-                    st = k_apply_param_gate(w, g, params, n_params, -1.0);
-                else
-                    st = k_apply_unfused(w, g);
-                if (st != QS_OK) break;
-            }
+            st = run_small(w, rev[c], params, n_params, /*param_sign=*/-1.0, gpart);
         } else {
             st = run_tiled(w, rev[c], params, n_params, /*force_bit=*/n, gpart, /*param_sign=*/-1.0);
         }

@@ -22,8 +22,6 @@ struct GradReduceP {
 
 qs_status k_dot(const StateView &a, const StateView &b, double *scratch, size_t scratch_doubles, double *out,
                 cudaStream_t st);
-// gradient op on a small (phi, lambda) state: out[b] for every member b
-qs_status k_grad_small(qs_state *w, const LGate &g, double *out);
 qs_status k_grad_reduce(const double *part, const GradReduceP &p, int n_param_rows, int batch, double *grad,
                         cudaStream_t st);
 

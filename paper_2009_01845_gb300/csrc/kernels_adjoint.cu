@@ -127,46 +127,4 @@ qs_status k_grad_reduce(const double *part, const GradReduceP &p, int n_param_ro
     return QS_OK;
 }
 
-// ------------------------------------------------------------------ small states
-// Gradient op for states too small for the sweep's tiles: one block per member
-// sums Im<lambda|P|phi> (see adjoint.cpp) over the member and writes out[b].
-template <typename R>
-__global__ void __launch_bounds__(256) grad_small_kernel(const V<R> *__restrict__ psi, int n, int gen, int tbit,
-                                                         uint64_t req, double *__restrict__ out) {
-    const int b = blockIdx.x;
-    const uint64_t half = 1ull << n;
-    const V<R> *ph = psi + ((uint64_t)b << (n + 1));
-    const V<R> *la = ph + half;
-    double acc = 0.0;
-    for (uint64_t x = threadIdx.x; x < half; x += blockDim.x) {
-        if ((x & req) != req) continue;
-        const bool tb = (x >> tbit) & 1ull;
-        const uint64_t xp = (gen == 0 || gen == 1) ? (x ^ (1ull << tbit)) : x;
-        const V<R> f = ph[xp], l = la[x];
-        const double im = (double)l.x * f.y - (double)l.y * f.x;
-        const double re = (double)l.x * f.x + (double)l.y * f.y;
-        if (gen == 0) acc += im;
-        else if (gen == 1) acc += tb ? re : -re;
-        else if (gen == 2) acc += tb ? -im : im;
-        else acc += im;
-    }
-    const double2 r = block_sum2_adj(acc, 0.0);
-    if (threadIdx.x == 0) out[b] = r.x;
-}
-
-qs_status k_grad_small(qs_state *w, const LGate &g, double *out) {
-    uint64_t req = g.cmask;
-    if (g.grad_gen == 3)
-        for (int j = 0; j < g.k; ++j) req |= 1ull << g.tbit[j];
-    ProfScope _ps(w->stream, KC_ADJOINT);
-    if (w->dtype == QS_C64)
-        grad_small_kernel<float><<<w->batch, 256, 0, w->stream>>>((const float2 *)w->data, w->n - 1, g.grad_gen,
-                                                                  g.tbit[0], req, out);
-    else
-        grad_small_kernel<double><<<w->batch, 256, 0, w->stream>>>((const double2 *)w->data, w->n - 1, g.grad_gen,
-                                                                   g.tbit[0], req, out);
-    QS_CUDA_TRY(cudaGetLastError());
-    return QS_OK;
-}
-
 }  // namespace qsim

@@ -4,6 +4,7 @@
 
 #include "fused.h"
 #include "plan.h"
+#include "small.h"
 #include "tiled.h"
 
 #include <algorithm>
@@ -88,6 +89,7 @@ static qs_status diag_factor(qs_state *s, const TrotterTerms &tt, double w0, dou
 // exp(-i dt X(s)) = prod_q RX(2 dt a_q(s)), RX(th) = exp(-i th X / 2)
 static qs_status x_layer(qs_state *s, const TrotterTerms &tt, double sv, double dt) {
     const int n = s->n;
+    std::vector<LGate> layer;
     for (int q = 0; q < n; ++q) {
         const double a = (1.0 - sv) * tt.a0[q] + sv * tt.a1[q];
         if (a == 0.0) continue;
@@ -100,8 +102,10 @@ static qs_status x_layer(qs_state *s, const TrotterTerms &tt, double sv, double 
         g.params[0] = 2.0 * dt * a;
         LGate lg;
         QS_TRY(lower_gate(n, g, &lg));
-        QS_TRY(k_apply_unfused(s, lg));
+        layer.push_back(std::move(lg));
     }
+    if (small_state(s)) return run_small(s, layer, nullptr, 0);
+    for (const LGate &lg : layer) QS_TRY(k_apply_unfused(s, lg));
     return QS_OK;
 }
 

@@ -22,6 +22,7 @@
 
 #include "plan.h"
 #include "prof.h"
+#include "small.h"
 #include "tiled.h"
 
 namespace qsim {
@@ -1320,13 +1321,7 @@ qs_status run_tiled(qs_state *s, const std::vector<LGate> &G, const double *para
             set_error("adjoint sweep needs n + 1 >= %d", k);
             return QS_ERR_UNSUPPORTED;
         }
-        for (const LGate &g : G) {
-            if (g.param_index >= 0)
-                QS_TRY(k_apply_param_gate(s, g, params, n_params));
-            else
-                QS_TRY(k_apply_unfused(s, g));
-        }
-        return QS_OK;
+        return run_small(s, G, params, n_params, param_sign);
     }
     const int nh = k - kTileLaneBits;  // chosen high tile bits
     const uint64_t force = force_bit >= 0 ? (1ull << force_bit) : 0ull;
