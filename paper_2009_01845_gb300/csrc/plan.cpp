@@ -38,6 +38,7 @@ qs_status run_gates(qs_state *s, std::vector<LGate> &gates, int mode, const qs_o
     case QS_MODE_AUTO:
     case QS_MODE_TILED:
     default:
+        if (small_state(s)) return run_small(s, gates, params_dev, n_params);
         return run_tiled(s, gates, params_dev, n_params);
     }
 }

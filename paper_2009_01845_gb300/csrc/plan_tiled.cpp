@@ -22,7 +22,6 @@
 
 #include "plan.h"
 #include "prof.h"
-#include "small.h"
 #include "tiled.h"
 
 namespace qsim {
@@ -1321,7 +1320,13 @@ qs_status run_tiled(qs_state *s, const std::vector<LGate> &G, const double *para
             set_error("adjoint sweep needs n + 1 >= %d", k);
             return QS_ERR_UNSUPPORTED;
         }
-        return run_small(s, G, params, n_params, param_sign);
+        for (const LGate &g : G) {
+            if (g.param_index >= 0)
+                QS_TRY(k_apply_param_gate(s, g, params, n_params));
+            else
+                QS_TRY(k_apply_unfused(s, g));
+        }
+        return QS_OK;
     }
     const int nh = k - kTileLaneBits;  // chosen high tile bits
     const uint64_t force = force_bit >= 0 ? (1ull << force_bit) : 0ull;
