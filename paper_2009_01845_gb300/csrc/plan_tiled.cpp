@@ -288,6 +288,26 @@ static std::vector<Entry> build_entries(const std::vector<LGate> &G, const std::
     return base;
 }
 
+// The non-factor entries of build_entries, for their needed bits alone: the
+// gates that stay gates, and the one-qubit gates that hold a rotation.
+static std::vector<Entry> stage_entries(const std::vector<LGate> &G, const std::vector<GClass> &cls,
+                                        const std::vector<int> &slot, const std::vector<int> &gates) {
+    std::vector<Entry> base;
+    base.reserve(gates.size());
+    for (int gi : gates) {
+        const LGate &g = G[gi];
+        const GClass c = cls[gi];
+        const bool fixed = slot[gi] < 0, plain = fixed && g.cmask == 0;
+        if ((plain && c == G_DIAG1) || (fixed && c == G_PHASE)) continue;
+        Entry e{plain && c == G_DENSE1 ? E_ROT : E_GATE};
+        if (e.kind == E_ROT && std::abs(g.m[2]) == 0.0) continue;
+        e.gi = gi;
+        e.bit = g.tbit[0];
+        base.push_back(std::move(e));
+    }
+    return base;
+}
+
 // slot[i]: per-member table slot of gate i (batched parameters) or -1.
 // Emits one tiled pass for the gates pp.gates; *fits = false (nothing launched)
 // when the pass exceeds the descriptor's capacity.
@@ -359,7 +379,8 @@ template <typename R> static void set_transpose(const TileStage &a, TileStage &b
 template <typename R>
 static qs_status emit_and_run(qs_state *s, const std::vector<LGate> &G, const std::vector<GClass> &cls,
                               const std::vector<int> &slot, uint32_t pm_stride, const PassPlan &pp,
-                              int force_bit, double *gpart, bool *fits, int *dry_stages = nullptr) {
+                              int force_bit, double *gpart, bool *fits, int *dry_stages = nullptr,
+                              bool count_only = false) {
     const int n = s->n;
     const int RB = TileCfg<R>::RB;
     const int k = RB + kTileLaneBits + TileCfg<R>::WB;
@@ -379,7 +400,8 @@ static qs_status emit_and_run(qs_state *s, const std::vector<LGate> &G, const st
     // register bit, as the gradient ops require.)
     const bool free_lanes = true;
     std::vector<FactorSpan> facs;
-    const std::vector<Entry> base = build_entries(G, cls, slot, pp.gates, free_lanes, &facs);
+    const std::vector<Entry> base = count_only ? stage_entries(G, cls, slot, pp.gates)
+                                               : build_entries(G, cls, slot, pp.gates, free_lanes, &facs);
     // needed local register bits of an entry
     auto need_of = [&](const Entry &e) {
         uint64_t nb = 0;
@@ -392,8 +414,7 @@ static qs_status emit_and_run(qs_state *s, const std::vector<LGate> &G, const st
         }
         if (e.kind == E_ROT && (free_lanes || e.bit >= kTileLaneBits)) nb = 1ull << e.bit;
         uint32_t l = 0;
-        for (int b = 0; b < 64; ++b)
-            if ((nb >> b) & 1ull) l |= 1u << loc_of[b];
+        for (; nb; nb &= nb - 1) l |= 1u << loc_of[__builtin_ctzll(nb)];
         return l;
     };
     // the stage choices below read needl/ne: first over the entries without
@@ -405,11 +426,15 @@ static qs_status emit_and_run(qs_state *s, const std::vector<LGate> &G, const st
     for (int i = 0; i < ne; ++i) needl[i] = need_of(base[i]);
     const uint32_t force_loc = force_bit >= 0 ? (1u << loc_of[force_bit]) : 0u;
     const uint32_t low5 = (1u << kTileLaneBits) - 1u;
-    auto next_use = [&](int from, int lb) {
-        for (int i = from; i < ne; ++i)
-            if ((needl[i] >> lb) & 1u) return i;
-        return std::numeric_limits<int>::max();
+    // next_use[i * k + lb]: the first entry from i on that needs local bit lb
+    std::vector<int> next_use;
+    auto index_uses = [&]() {
+        next_use.assign((size_t)(ne + 1) * k, std::numeric_limits<int>::max());
+        for (int i = ne - 1; i >= 0; --i)
+            for (int lb = 0; lb < k; ++lb)
+                next_use[(size_t)i * k + lb] = ((needl[i] >> lb) & 1u) ? i : next_use[(size_t)(i + 1) * k + lb];
     };
+    index_uses();
     // register set: forced bits plus the candidate bits used soonest from entry
     // `from` on (furthest-next-use eviction)
     auto choose = [&](int from, uint32_t forced, uint32_t candidates) {
@@ -417,7 +442,7 @@ static qs_status emit_and_run(qs_state *s, const std::vector<LGate> &G, const st
         std::vector<std::pair<int, int>> rank;  // (next use, local bit)
         for (int lb = 0; lb < k; ++lb) {
             if (((forced >> lb) & 1u) || !((candidates >> lb) & 1u)) continue;
-            rank.push_back({next_use(from, lb), lb});
+            rank.push_back({next_use[(size_t)from * k + lb], lb});
         }
         std::sort(rank.begin(), rank.end());
         uint32_t r = forced;
@@ -453,6 +478,26 @@ static qs_status emit_and_run(qs_state *s, const std::vector<LGate> &G, const st
 
     const uint32_t low5_mask = (1u << kTileLaneBits) - 1u;
     const uint32_t high_bits = ((1u << k) - 1u) & ~low5_mask;
+
+    // Stages alone: diagonal blocks need no bits, so the stages open at the same
+    // entries with and without them (capacity is not checked here).
+    if (count_only) {
+        uint32_t c = choose(0, (ne ? needl[0] : 0u) & high_bits, high_bits);
+        uint32_t lanes = low5_mask;
+        int stages = 1;
+        for (int i = 0; i < ne; ++i) {
+            if ((needl[i] & ~c) == 0) continue;
+            c = choose(i, needl[i], (1u << k) - 1u);
+            lanes = 0;
+            for (int lb : lanes_for(i, c)) lanes |= 1u << lb;
+            ++stages;
+        }
+        const uint32_t sector_bits = sizeof(R) == 4 ? 3u : 1u;
+        if ((lanes & sector_bits) != sector_bits) ++stages;
+        *dry_stages = stages;
+        *fits = stages <= kTileMaxStages;
+        return QS_OK;
+    }
 
     // Diagonal blocks. The register set in effect at every entry (a stage
     // opens at an entry whose needed bits are not all registers). Costs in
@@ -495,9 +540,8 @@ static qs_status emit_and_run(qs_state *s, const std::vector<LGate> &G, const st
         // cost of factor f at a cut with register set regs; *walk: needs the phase walk
         auto cost = [&](const Factor &f, uint32_t regs, bool *walk) {
             int nr = 0, nt = 0, no = 0;
-            const uint64_t m = factor_bits(f);
-            for (int b = 0; b < 64; ++b) {
-                if (!((m >> b) & 1ull)) continue;
+            for (uint64_t m = factor_bits(f); m; m &= m - 1) {
+                const int b = __builtin_ctzll(m);
                 const int lb = b < n ? loc_of[b] : -1;
                 if (lb < 0) ++no;
                 else if ((regs >> lb) & 1u) ++nr;
@@ -514,6 +558,18 @@ static qs_status emit_and_run(qs_state *s, const std::vector<LGate> &G, const st
             if (sign) return 10;
             return nr >= 2 ? 60 : 25;
         };
+        // cost of factor j at cut q, each computed once
+        std::vector<int> memo((size_t)nf * (nbase + 1), -1);
+        auto cost_at = [&](int j, int q, bool *walk) {
+            int &m = memo[(size_t)j * (nbase + 1) + q];
+            if (m < 0) {
+                bool w;
+                const int c = cost(facs[j].f, reg_base[q], &w);
+                m = 2 * c + (w ? 1 : 0);
+            }
+            *walk = (m & 1) != 0;
+            return m >> 1;
+        };
         std::vector<int> where(nf, -1), fc(nf, 0);
         std::vector<char> fw(nf, 0);
         for (int j = 0; j < nf; ++j) {
@@ -521,7 +577,7 @@ static qs_status emit_and_run(qs_state *s, const std::vector<LGate> &G, const st
             for (int p = facs[j].left + 1; p <= facs[j].right; ++p) {
                 if (!open[p]) continue;
                 bool w;
-                const int cc = cost(facs[j].f, reg_base[p], &w);
+                const int cc = cost_at(j, p, &w);
                 if (cc < bc) {
                     bc = cc;
                     where[j] = p;
@@ -535,15 +591,16 @@ static qs_status emit_and_run(qs_state *s, const std::vector<LGate> &G, const st
             std::vector<int> walkers(nbase + 1, 0);
             for (int j = 0; j < nf; ++j) walkers[where[j]] += fw[j];
             int best_q = -1, best_delta = 0;
+            std::vector<int> left_walkers;
             for (int q = 0; q <= nbase; ++q) {
                 if (!cand[q] || open[q]) continue;
                 int delta = 0;
                 bool q_walks = false;
-                std::vector<int> left_walkers = walkers;
+                left_walkers = walkers;
                 for (int j = 0; j < nf; ++j) {
                     if (!(facs[j].left < q && q <= facs[j].right)) continue;
                     bool w;
-                    const int cc = cost(facs[j].f, reg_base[q], &w);
+                    const int cc = cost_at(j, q, &w);
                     if (cc >= fc[j]) continue;
                     delta += cc - fc[j];
                     q_walks = q_walks || w;
@@ -560,7 +617,7 @@ static qs_status emit_and_run(qs_state *s, const std::vector<LGate> &G, const st
             for (int j = 0; j < nf; ++j) {
                 if (!(facs[j].left < best_q && best_q <= facs[j].right)) continue;
                 bool w;
-                const int cc = cost(facs[j].f, reg_base[best_q], &w);
+                const int cc = cost_at(j, best_q, &w);
                 if (cc >= fc[j]) continue;
                 where[j] = best_q;
                 fc[j] = cc;
@@ -580,6 +637,7 @@ static qs_status emit_and_run(qs_state *s, const std::vector<LGate> &G, const st
         ne = (int)ent.size();
         needl.assign(ne, 0u);
         for (int i = 0; i < ne; ++i) needl[i] = need_of(ent[i]);
+        index_uses();
     }
     // a diagonal block is placed in the stage of the next non-block entry
     // (that stage opens before the block)
@@ -656,8 +714,8 @@ static qs_status emit_and_run(qs_state *s, const std::vector<LGate> &G, const st
         *mr = 0;
         *mt = 0;
         *mo = 0;
-        for (int b = 0; b < 64; ++b) {
-            if (!((gm >> b) & 1ull)) continue;
+        for (; gm; gm &= gm - 1) {
+            const int b = __builtin_ctzll(gm);
             const int lb = b < n ? loc_of[b] : -1;
             if (lb < 0) {
                 *mo |= 1ull << b;
@@ -1411,35 +1469,50 @@ qs_status run_tiled(qs_state *s, const std::vector<LGate> &G, const double *para
         // complete the tile with unused high bits
         for (int b = kTileLaneBits; b < n && __builtin_popcountll(pp.high) < nh; ++b) pp.high |= 1ull << b;
         // order: the fewest stages among the queue order and two orders that
-        // reverse alternate runs of mutually commuting gates
-        if (pp.gates.size() > 1) {
-            std::vector<std::vector<int>> cand = run_orders(G, cls, pp.gates);
-            int best = -1, best_stages = std::numeric_limits<int>::max();
+        // reverse alternate runs of mutually commuting gates. Stages are counted
+        // without emitting; only where the chosen order exceeds the descriptor's
+        // capacity are the candidates emitted to find the best that fits
+        auto emit = [&](const PassPlan &q, bool *fits, int *stages, bool count_only) {
+            return s->dtype == QS_C64
+                       ? emit_and_run<float>(s, G, cls, slot, pm_stride, q, force_bit, gpart, fits, stages, count_only)
+                       : emit_and_run<double>(s, G, cls, slot, pm_stride, q, force_bit, gpart, fits, stages, count_only);
+        };
+        std::vector<std::vector<int>> cand;
+        auto best_order = [&](bool count_only, int *out) -> qs_status {
+            int best_stages = std::numeric_limits<int>::max();
+            *out = -1;
             for (size_t c = 0; c < cand.size(); ++c) {
-                PassPlan q = pp;
+                PassPlan q;
+                q.high = pp.high;
                 q.gates = cand[c];
                 bool fits = true;
                 int stages = 0;
-                if (s->dtype == QS_C64)
-                    QS_TRY(emit_and_run<float>(s, G, cls, slot, pm_stride, q, force_bit, gpart, &fits, &stages));
-                else
-                    QS_TRY(emit_and_run<double>(s, G, cls, slot, pm_stride, q, force_bit, gpart, &fits, &stages));
+                QS_TRY(emit(q, &fits, &stages, count_only));
                 if (fits && stages < best_stages) {
                     best_stages = stages;
-                    best = (int)c;
+                    *out = (int)c;
                 }
             }
-            if (best > 0) pp.gates = cand[best];
+            return QS_OK;
+        };
+        int order = -1;
+        if (pp.gates.size() > 1) {
+            cand = run_orders(G, cls, pp.gates);
+            QS_TRY(best_order(true, &order));
+            if (order > 0) pp.gates = cand[order];
         }
         // emit; a pass over the descriptor's capacity is retried with a prefix of
         // its gates (a prefix keeps every dependency)
         while (true) {
             bool fits = true;
-            if (s->dtype == QS_C64)
-                QS_TRY(emit_and_run<float>(s, G, cls, slot, pm_stride, pp, force_bit, gpart, &fits));
-            else
-                QS_TRY(emit_and_run<double>(s, G, cls, slot, pm_stride, pp, force_bit, gpart, &fits));
+            QS_TRY(emit(pp, &fits, nullptr, false));
             if (fits) break;
+            if (!cand.empty()) {
+                QS_TRY(best_order(false, &order));
+                pp.gates = cand[std::max(order, 0)];
+                cand.clear();
+                if (order >= 0) continue;
+            }
             if (pp.gates.size() <= 1) {
                 set_error("tiled planner cannot fit a single gate");
                 return QS_ERR_CUDA;

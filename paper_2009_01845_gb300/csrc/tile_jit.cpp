@@ -97,6 +97,7 @@ struct JitGlobal {
     std::vector<std::thread> workers;
     int busy = 0;
     int entries = 0;
+    int folded = 0;  // entries with their values compiled in
     std::unordered_map<uint64_t, int> full_seen;  // launches per exact pass (by hash)
     bool stop = false;
     std::atomic<int> policy{-1};
@@ -153,13 +154,23 @@ int policy_now() {
     return p;
 }
 
-uint64_t fnv(const unsigned char *b, size_t n) {
-    uint64_t h = 1469598103934665603ull;
-    for (size_t i = 0; i < n; ++i) {
-        h ^= b[i];
-        h *= 1099511628211ull;
-    }
-    return h;
+// Hash of a key (whole keys are compared on a match): FNV over 8-byte words in
+// four interleaved lanes (a key is about 24 KB and is hashed for every launch:
+// 3 us, 30 us a byte at a time).
+uint64_t key_hash(const unsigned char *b, size_t n) {
+    uint64_t h[4] = {1469598103934665603ull, 0x9e3779b97f4a7c15ull, 0xc2b2ae3d27d4eb4full, 0x165667b19e3779f9ull};
+    size_t i = 0;
+    for (; i + 32 <= n; i += 32)
+        for (int j = 0; j < 4; ++j) {
+            uint64_t w;
+            std::memcpy(&w, b + i + 8 * j, 8);
+            h[j] = (h[j] ^ w) * 1099511628211ull;
+            h[j] ^= h[j] >> 29;
+        }
+    for (; i < n; ++i) h[0] = (h[0] ^ b[i]) * 1099511628211ull;
+    uint64_t r = 0;
+    for (int j = 0; j < 4; ++j) r = (r ^ h[j]) * 1099511628211ull ^ (r >> 31);
+    return r;
 }
 
 // ------------------------------------------------------------------ source generation
@@ -470,31 +481,32 @@ qs_status tile_jit_launch_t(qs_state *s, const TileParams<R> &p, bool *launched)
     // descriptor with its run-time pointers and the Ising op's tau (which only
     // the table kernel reads) cleared; the structure key also clears the
     // values (matrix entries, diagonal factors)
-    std::vector<unsigned char> full(1 + sizeof(TileParams<R>));
-    full[0] = kTypeCode<R> | kKeyFolded;
-    {
-        TileParams<R> &k = *reinterpret_cast<TileParams<R> *>(full.data() + 1);
-        std::memcpy(&k, &p, sizeof(p));
-        k.pmat = nullptr;
-        k.gpart = nullptr;
-        k.ising = nullptr;
-        k.ising_thr = nullptr;
+    static thread_local std::vector<unsigned char> full, key;  // reused between launches
+    const size_t bytes = 1 + sizeof(TileParams<R>);
+    auto fill = [&](std::vector<unsigned char> &dst, unsigned char flags) {
+        dst.resize(bytes);
+        dst[0] = flags;
+        unsigned char *k = dst.data() + 1;
+        auto clear = [&](const void *field, size_t n) {
+            std::memset(k + ((const unsigned char *)field - (const unsigned char *)&p), 0, n);
+        };
+        std::memcpy(k, &p, sizeof(p));
+        clear(&p.pmat, sizeof(p.pmat));
+        clear(&p.gpart, sizeof(p.gpart));
+        clear(&p.ising, sizeof(p.ising));
+        clear(&p.ising_thr, sizeof(p.ising_thr));
         for (int o = 0; o < kTileMaxOps; ++o)
-            if (k.op[o].type == TOP_ISING) k.op[o].tmask = 0;
-    }
-    std::vector<unsigned char> key(full);
-    key[0] = kTypeCode<R>;
-    {
-        TileParams<R> &k = *reinterpret_cast<TileParams<R> *>(key.data() + 1);
-        std::memset(k.mat, 0, sizeof(k.mat));
+            if (p.op[o].type == TOP_ISING) clear(&p.op[o].tmask, sizeof(p.op[o].tmask));
+        if (flags & kKeyFolded) return;
+        clear(p.mat, sizeof(p.mat));
         for (int f = 0; f < kTileMaxDFac; ++f) {
-            std::memset(&k.dfac[f].v0, 0, sizeof(k.dfac[f].v0));
-            std::memset(&k.dfac[f].v1, 0, sizeof(k.dfac[f].v1));
-            std::memset(&k.dfac[f].v2, 0, sizeof(k.dfac[f].v2));
+            clear(&p.dfac[f].v0, sizeof(p.dfac[f].v0));
+            clear(&p.dfac[f].v1, sizeof(p.dfac[f].v1));
+            clear(&p.dfac[f].v2, sizeof(p.dfac[f].v2));
         }
-    }
-    const uint64_t h = fnv(key.data(), key.size());
-    const uint64_t hf = fnv(full.data(), full.size());
+    };
+    fill(key, kTypeCode<R>);
+    const uint64_t h = key_hash(key.data(), bytes);
     std::shared_ptr<JitEntry> e;
     bool compile_here = false;
     {
@@ -509,9 +521,11 @@ qs_status tile_jit_launch_t(qs_state *s, const TileParams<R> &p, bool *launched)
         // once the exact pass has been launched twice (counted by hash; the
         // entry itself compares whole keys)
         std::shared_ptr<JitEntry> ef;
-        if (policy != QS_JIT_OFF) {
+        if (fold || g.folded > 0) {
             // existing folded kernels are used whatever the flag; new ones are
             // made only under QS_JIT_FOLD
+            fill(full, kTypeCode<R> | kKeyFolded);
+            const uint64_t hf = key_hash(full.data(), bytes);
             auto fb = g.table.find(hf);
             if (fb != g.table.end())
                 for (auto &c : fb->second)
@@ -521,6 +535,7 @@ qs_status tile_jit_launch_t(qs_state *s, const TileParams<R> &p, bool *launched)
                     }
             if (!ef && fold && !capturing && !g.stop && ++g.full_seen[hf] >= 2 && g.entries < kMaxEntries) {
                 ++g.entries;
+                ++g.folded;
                 ef = std::make_shared<JitEntry>();
                 ef->key = full;
                 ef->type = kTypeCode<R>;
@@ -556,7 +571,7 @@ qs_status tile_jit_launch_t(qs_state *s, const TileParams<R> &p, bool *launched)
             }
             ++g.entries;
             e = std::make_shared<JitEntry>();
-            e->key = std::move(key);
+            e->key = key;
             e->type = kTypeCode<R>;
             bucket.push_back(e);
         }
