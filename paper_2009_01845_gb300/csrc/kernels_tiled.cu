@@ -24,81 +24,88 @@ namespace qsim {
 template <typename R> qs_status tile_jit_launch_t(qs_state *s, const TileParams<R> &p, bool *launched);
 
 // The Ising op's tables (see ising_thr_stride), per member (blockIdx.y), in
-// FP64: block 0, one thread per thread pattern (lane bits, then warp bits), the
-// pattern's coupling energy and fields, and the register-pair energies; blocks
-// 1.., one thread per tile, the fields of the outside bits on the tile bits and
-// the outside energy. Every energy x is stored as exp(-i tau x).
-__global__ void __launch_bounds__(256) ising_table_kernel(const __grid_constant__ IsingTabP tp) {
-    const int member = blockIdx.y, tid = threadIdx.x;
-    const int nq = tp.nq;
+// FP64, one thread per entry in the table's own order: for every thread pattern
+// (lane bits, then warp bits) its coupling energy with the fields it puts on the
+// register bits, then each of those fields; the register-pair energies; for
+// every tile the fields of the outside bits on the tile bits and the outside
+// energy. Every energy x is stored as exp(-i tau x). Bound by the FP64 pipe (2
+// operations per clock and SM), so the entries are spread over as many SMs as
+// there are: 64 threads a CTA. A thread per pattern or per tile, 256 a CTA (all
+// patterns of a member on one SM), took 30 us at n = 16 .. 22; 20 steps of two
+// 24-qubit instances, complex64: 6.74 -> 6.16 ms.
+constexpr int kIsingTabThreads = 64;
+
+__global__ void __launch_bounds__(kIsingTabThreads) ising_table_kernel(const __grid_constant__ IsingTabP tp) {
+    const int member = blockIdx.y, nq = tp.nq;
     const double *J = tp.ising + (size_t)member * tp.ising_stride;
     const double *hv = J + (size_t)nq * nq;
     double2 *base = reinterpret_cast<double2 *>(tp.out + (size_t)member * tp.stride);
-    auto put = [&](double2 *dst, double x) {
-        if (tp.single) {
-            const V<float> v = expi<float>(-tp.tau * x);
-            *dst = make_double2(v.x, v.y);
-        } else {
-            const V<double> v = expi<double>(-tp.tau * x);
-            *dst = make_double2(v.x, v.y);
-        }
-    };
-    if (blockIdx.x == 0) {
-        double z[kTileLaneBits + kTileMaxWarpBits];
-        for (int i = 0; i < tp.tb; ++i) z[i] = ((tid >> i) & 1) ? -1.0 : 1.0;
-        double e = 0.0;
-        for (int i = 0; i < tp.tb; ++i)
-            for (int j = i + 1; j < tp.tb; ++j) e += J[tp.tg[i] * nq + tp.tg[j]] * z[i] * z[j];
-        double2 *row = base + (size_t)tid * (1 + tp.rb);
-        double wsum = 0.0;
-        for (int j = 0; j < tp.rb; ++j) {
+    const uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const uint64_t patterns = (uint64_t)(1 + tp.rb) << tp.tb, pairs = patterns + (1u << tp.rb);
+    if (i >= pairs + ((uint64_t)(tp.k + 1) << tp.n_free)) return;
+    double x;
+    if (i < patterns) {
+        const int tid = (int)(i / (1 + tp.rb)), c = (int)(i % (1 + tp.rb));
+        auto z = [&](int b) { return ((tid >> b) & 1) ? -1.0 : 1.0; };
+        auto field = [&](int j) {  // on register bit j
             double w = 0.0;
-            for (int i = 0; i < tp.tb; ++i) w += J[tp.rg[j] * nq + tp.tg[i]] * z[i];
-            wsum += w;
-            put(&row[1 + j], -2.0 * w);
+            for (int b = 0; b < tp.tb; ++b) w += J[tp.rg[j] * nq + tp.tg[b]] * z(b);
+            return w;
+        };
+        if (c > 0) {
+            x = -2.0 * field(c - 1);
+        } else {
+            double e = 0.0, wsum = 0.0;
+            for (int a = 0; a < tp.tb; ++a)
+                for (int b = a + 1; b < tp.tb; ++b) e += J[tp.tg[a] * nq + tp.tg[b]] * z(a) * z(b);
+            for (int j = 0; j < tp.rb; ++j) wsum += field(j);
+            x = e + wsum;
         }
-        put(&row[0], e + wsum);
-        if (tid < (1 << tp.rb)) {
-            double q = 0.0;
-            for (int i = 0; i < tp.rb; ++i)
-                for (int j = i + 1; j < tp.rb; ++j) {
-                    const double c = J[tp.rg[i] * nq + tp.rg[j]];
-                    q += (((tid >> i) ^ (tid >> j)) & 1) ? -c : c;
-                }
-            put(base + (size_t)blockDim.x * (1 + tp.rb) + tid, q);
+    } else if (i < pairs) {
+        const int r = (int)(i - patterns);
+        x = 0.0;
+        for (int a = 0; a < tp.rb; ++a)
+            for (int b = a + 1; b < tp.rb; ++b) {
+                const double c = J[tp.rg[a] * nq + tp.rg[b]];
+                x += (((r >> a) ^ (r >> b)) & 1) ? -c : c;
+            }
+    } else {
+        // bit o of a tile's number is the outside bit og[o]
+        const uint64_t t = (i - pairs) / (tp.k + 1);
+        const int c = (int)((i - pairs) % (tp.k + 1));
+        auto sum = [&](int g, int from) {  // h and the couplings of bit g with the outside bits from `from` on
+            double acc = hv[g];
+            for (int o = from; o < tp.n_free; ++o) acc += ((t >> o) & 1ull) ? -J[g * nq + tp.og[o]] : J[g * nq + tp.og[o]];
+            return acc;
+        };
+        if (c < tp.k) {
+            x = sum(tp.gb[c], 0);
+        } else {
+            x = hv[nq];
+            for (int o = 0; o < tp.n_free; ++o) x += (((t >> o) & 1ull) ? -1.0 : 1.0) * sum(tp.og[o], o + 1);
         }
-        return;
     }
-    const uint64_t t = (uint64_t)(blockIdx.x - 1) * blockDim.x + tid;
-    if (t >= (1ull << tp.n_free)) return;
-    const uint64_t tbase = expand_bits(t, tp.tins);  // the tile's outside bits
-    uint64_t tmask = 0;
-    for (int i = 0; i < tp.k; ++i) tmask |= 1ull << tp.gb[i];
-    double2 *row = base + (size_t)blockDim.x * (1 + tp.rb) + (1 << tp.rb) + t * (tp.k + 1);
-    for (int i = 0; i < tp.k; ++i) {
-        const int g = tp.gb[i];
-        double acc = hv[g];
-        for (int o = 0; o < nq; ++o)
-            if (!((tmask >> o) & 1ull)) acc += ((tbase >> o) & 1ull) ? -J[g * nq + o] : J[g * nq + o];
-        put(&row[i], acc);
+    if (tp.single) {
+        const V<float> v = expi<float>(-tp.tau * x);
+        base[i] = make_double2(v.x, v.y);
+    } else {
+        const V<double> v = expi<double>(-tp.tau * x);
+        base[i] = make_double2(v.x, v.y);
     }
-    double eo = hv[nq];
-    for (int o = 0; o < nq; ++o) {
-        if ((tmask >> o) & 1ull) continue;
-        const double zo = ((tbase >> o) & 1ull) ? -1.0 : 1.0;
-        double r = hv[o];
-        for (int o2 = o + 1; o2 < nq; ++o2)
-            if (!((tmask >> o2) & 1ull)) r += ((tbase >> o2) & 1ull) ? -J[o * nq + o2] : J[o * nq + o2];
-        eo += zo * r;
-    }
-    put(&row[tp.k], eo);
 }
 
-qs_status k_ising_table(qs_state *s, const IsingTabP &tp) {
-    if (tp.members <= 0) return QS_OK;
+qs_status k_ising_table(qs_state *s, const IsingTabP &in) {
+    if (in.members <= 0) return QS_OK;
     ProfScope _ps(s->stream, KC_TROTTER_DIAG);
-    const dim3 grid(1 + (unsigned)(((1ull << tp.n_free) + 255) / 256), (unsigned)tp.members);
-    ising_table_kernel<<<grid, 256, 0, s->stream>>>(tp);
+    IsingTabP tp = in;
+    uint64_t tile = 0;
+    for (int i = 0; i < tp.k; ++i) tile |= 1ull << tp.gb[i];
+    int no = 0;
+    for (int b = 0; b < tp.nq; ++b)
+        if (!((tile >> b) & 1ull)) tp.og[no++] = (int8_t)b;
+    const uint64_t entries = ((uint64_t)(1 + tp.rb) << tp.tb) + (1u << tp.rb) + ((uint64_t)(tp.k + 1) << tp.n_free);
+    const dim3 grid((unsigned)((entries + kIsingTabThreads - 1) / kIsingTabThreads), (unsigned)tp.members);
+    ising_table_kernel<<<grid, kIsingTabThreads, 0, s->stream>>>(tp);
     QS_CUDA_TRY(cudaGetLastError());
     return QS_OK;
 }

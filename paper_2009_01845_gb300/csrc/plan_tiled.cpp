@@ -1262,7 +1262,6 @@ static qs_status emit_and_run(qs_state *s, const std::vector<LGate> &G, const st
                 tp.k = k;
                 tp.n_free = P.n_free;
                 for (int i = 0; i < k; ++i) tp.gb[i] = (int8_t)P.gbit[i];
-                tp.tins = P.tins;
                 std::memcpy(&tp.tau, &op.tmask, sizeof(double));
                 tp.ising = s->itab;
                 tp.ising_stride = s->ising_stride;

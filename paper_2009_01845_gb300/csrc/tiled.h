@@ -227,14 +227,12 @@ __host__ __device__ constexpr size_t tile_smem_bytes(int k, int n_stages) {
 
 // Inputs of the Ising-table kernel for one op: global bits of the stage's
 // thread bits (lanes 0..4, then warps) and register bits, the pass's tile bits
-// (k of them, global positions gb, inserted into a tile number by tins), tau,
-// and where the op's tables start.
+// (k of them, global positions gb), tau, and where the op's tables start.
 struct IsingTabP {
     int8_t tg[kTileLaneBits + kTileMaxWarpBits];
     int8_t rg[6];
     int8_t gb[16];
     int tb, rb, k, n_free;
-    InsertBits tins;
     double tau;
     const double *ising;
     uint32_t ising_stride;
@@ -243,6 +241,7 @@ struct IsingTabP {
     uint32_t stride;   // doubles per member
     int members;
     int single;        // the state is complex64: sin and cos in FP32 (of the FP64-reduced angle)
+    int8_t og[QS_MAX_QUBITS];  // outside bits, ascending (filled by the launch)
 };
 
 // The Ising op's tables, per member, as (cos, sin) pairs of exp(-i tau x):
