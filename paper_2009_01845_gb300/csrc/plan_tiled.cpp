@@ -5,12 +5,12 @@
 //   * its dense targets fit in the tile (5 lane bits + k-5 chosen bits); diagonal
 //     gates need no tile bits at all, since a tile knows every index bit of
 //     every amplitude it holds.
-// A gate the tile cannot express (dense on 3+ qubits, a 2-qubit dense gate
-// touching a lane bit, a general 2+-qubit diagonal, a batched parameter) is
-// applied by its own unfused pass when it reaches the front of the queue.
-// Within a pass, stages re-split the k-5 high tile bits between registers and
-// warps; the register set of a new stage is the needed bits plus the bits used
-// soonest afterwards (furthest-next-use eviction).
+// A gate the tile cannot express (dense on 3+ qubits, a general 2+-qubit
+// diagonal, for complex128 a SWAP of a lane bit) is applied by its own unfused
+// pass when it reaches the front of the queue. Within a pass, stages re-split
+// the tile's bits, lane bits included, between registers, lanes and warps; the
+// register set of a new stage is the needed bits plus the bits used soonest
+// afterwards (furthest-next-use eviction).
 #include <algorithm>
 #include <cstdio>
 #include <cstdlib>
@@ -34,7 +34,9 @@ namespace {
 
 enum GClass { G_PHASE, G_DIAG1, G_DENSE1, G_DENSE2, G_SWAP, G_GRAD, G_ISING, G_SINGLE };
 
-GClass classify(const LGate &g) {
+// low_swaps: SWAPs that touch a lane bit may run in a tile too (complex128 in
+// double-float keeps those in passes of their own, which move amplitudes exactly)
+GClass classify(const LGate &g, bool low_swaps) {
     if (g.kind == kKindGrad) return G_GRAD;
     if (g.kind == kKindIsing) return G_ISING;
     if (g.param_index >= 0) {
@@ -48,9 +50,10 @@ GClass classify(const LGate &g) {
     }
     if (g.phase_only) return G_PHASE;
     if (g.diagonal) return g.k == 1 ? G_DIAG1 : G_SINGLE;
-    if (g.is_swap) return (g.tbit[0] >= kTileLaneBits && g.tbit[1] >= kTileLaneBits) ? G_SWAP : G_SINGLE;
+    if (g.is_swap)
+        return low_swaps || (g.tbit[0] >= kTileLaneBits && g.tbit[1] >= kTileLaneBits) ? G_SWAP : G_SINGLE;
     if (g.k == 1) return G_DENSE1;
-    if (g.k == 2) return (g.tbit[0] >= kTileLaneBits && g.tbit[1] >= kTileLaneBits) ? G_DENSE2 : G_SINGLE;
+    if (g.k == 2) return G_DENSE2;
     return G_SINGLE;
 }
 
@@ -60,14 +63,15 @@ uint64_t qubit_bits(const LGate &g) {
     return m;
 }
 
-// high (non-lane) global bits a gate needs inside the tile
-uint64_t need_bits(const LGate &g, GClass c) {
-    if (c == G_DENSE1) return g.tbit[0] >= kTileLaneBits ? (1ull << g.tbit[0]) : 0;
-    if (c == G_GRAD && (g.grad_gen == GEN_X || g.grad_gen == GEN_Y))
-        return g.tbit[0] >= kTileLaneBits ? (1ull << g.tbit[0]) : 0;
+// global bits that must be register bits where a gate is applied
+uint64_t target_bits(const LGate &g, GClass c) {
+    if (c == G_DENSE1 || (c == G_GRAD && (g.grad_gen == GEN_X || g.grad_gen == GEN_Y))) return 1ull << g.tbit[0];
     if (c == G_DENSE2 || c == G_SWAP) return (1ull << g.tbit[0]) | (1ull << g.tbit[1]);
     return 0;
 }
+
+// the high (non-lane) ones: the tile has to include them
+uint64_t need_bits(const LGate &g, GClass c) { return target_bits(g, c) & ~((1ull << kTileLaneBits) - 1ull); }
 
 int mat_entries(GClass c) {
     switch (c) {
@@ -405,13 +409,7 @@ static qs_status emit_and_run(qs_state *s, const std::vector<LGate> &G, const st
     // needed local register bits of an entry
     auto need_of = [&](const Entry &e) {
         uint64_t nb = 0;
-        if (e.kind == E_GATE) {
-            const LGate &g = G[e.gi];
-            const GClass c = cls[e.gi];
-            nb = need_bits(g, c);
-            if (free_lanes && (c == G_DENSE1 || (c == G_GRAD && (g.grad_gen == GEN_X || g.grad_gen == GEN_Y))))
-                nb = 1ull << g.tbit[0];
-        }
+        if (e.kind == E_GATE) nb = target_bits(G[e.gi], cls[e.gi]);
         if (e.kind == E_ROT && (free_lanes || e.bit >= kTileLaneBits)) nb = 1ull << e.bit;
         uint32_t l = 0;
         for (; nb; nb &= nb - 1) l |= 1u << loc_of[__builtin_ctzll(nb)];
@@ -1388,7 +1386,8 @@ qs_status run_tiled(qs_state *s, const std::vector<LGate> &G, const double *para
     const int nh = k - kTileLaneBits;  // chosen high tile bits
     const uint64_t force = force_bit >= 0 ? (1ull << force_bit) : 0ull;
     std::vector<GClass> cls(G.size());
-    for (size_t i = 0; i < G.size(); ++i) cls[i] = classify(G[i]);
+    const bool low_swaps = s->dtype == QS_C64 || c128_fp64();
+    for (size_t i = 0; i < G.size(); ++i) cls[i] = classify(G[i], low_swaps);
     // per-member matrices of every batched-parameter gate, built once on the device
     std::vector<int> slot(G.size(), -1), spidx, skind;
     for (size_t i = 0; i < G.size(); ++i)
