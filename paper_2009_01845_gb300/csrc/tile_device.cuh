@@ -393,6 +393,85 @@ __device__ __forceinline__ void diag_block(V<R> *a, const TileParams<R> &p, cons
     }
 }
 
+// v negated where s is 0x80000000 (s is that or 0)
+template <typename R> __device__ __forceinline__ V<R> csign(V<R> v, uint32_t s) {
+    auto flip = [&](float x) { return __uint_as_float(__float_as_uint(x) ^ s); };
+    if constexpr (is_dd<R>) {
+        v.h = make_float2(flip(v.h.x), flip(v.h.y));
+        v.l = make_float2(flip(v.l.x), flip(v.l.y));
+    } else if constexpr (sizeof(R) == 4) {
+        v.x = flip(v.x);
+        v.y = flip(v.y);
+    } else {
+        v.x = __hiloint2double(__double2hiint(v.x) ^ (int)s, __double2loint(v.x));
+        v.y = __hiloint2double(__double2hiint(v.y) ^ (int)s, __double2loint(v.y));
+    }
+    return v;
+}
+
+// The sign factors of a diagonal block at register r, as a sign bit: NEG holds
+// the bits the block's factors may negate (bit j: the ratio of register bit j,
+// bit 7: the base), s[] their sign bits in this thread.
+template <int RB, uint32_t NEG> struct BlockSigns {
+    uint32_t s[RB], base;
+    template <typename R>
+    __device__ __forceinline__ BlockSigns(const TileParams<R> &p, const TileOp &op, uint64_t tbase, uint32_t lt) {
+        uint32_t neg = 0;
+        const int f0 = (int)op.mo;
+        for (int f = f0; f < f0 + op.tkind; ++f) {
+            const TileDFac<R> &d = p.dfac[f];
+            if ((tbase & d.mo) == d.mo && (lt & d.mt) == d.mt) neg ^= d.a;
+        }
+        base = (NEG & 0x80u) ? (neg & 0x80u) << 24 : 0u;
+#pragma unroll
+        for (int j = 0; j < RB; ++j) s[j] = ((NEG >> j) & 1u) ? (neg << (31 - j)) & 0x80000000u : 0u;
+    }
+    __device__ __forceinline__ uint32_t at(int r) const {
+        uint32_t v = base;
+#pragma unroll
+        for (int j = 0; j < RB; ++j)
+            if ((r >> j) & 1) v ^= s[j];
+        return v;
+    }
+};
+
+// A diagonal block (TOP_DBLOCK) whose only factors under thread or outside bits
+// are signs, in a specialised kernel: every register's phase is the same in all
+// threads up to its sign, so the 2^RB phases come from a table in the parameter
+// block, the uniform sign flips before the block folded in. One complex product
+// per register; the walk of diag_block takes two (base and ratios vary). A
+// complex64 block of 32 registers is 128 FMA-pipe instructions instead of 252, a
+// double-float one of 16 registers 16 complex products instead of 31.
+template <typename R, int RB, uint32_t NEG>
+__device__ __forceinline__ void diag_table(V<R> *a, const TileParams<R> &p, const V<R> *tab, const TileOp &op,
+                                           uint64_t tbase, uint32_t lt) {
+    const BlockSigns<RB, NEG> sg(p, op, tbase, lt);
+#pragma unroll
+    for (int r = 0; r < (1 << RB); ++r) a[r] = cmul<R>(a[r], csign<R>(tab[r], sg.at(r)));
+}
+
+// The same where every phase is +1 or -1 (bit r of `minus`: -1): signs alone,
+// in complex64 one paired product by +-1 for a register whose sign varies. Energy
+// and gradient of 10 RY and CZ layers at n = 18, 64 members, complex64: 3.28 ms
+// with the walk of diag_block for the CZ signs, 3.08 ms.
+template <typename R, int RB, uint32_t NEG>
+__device__ __forceinline__ void diag_signs(V<R> *a, const TileParams<R> &p, uint32_t minus, const TileOp &op,
+                                           uint64_t tbase, uint32_t lt) {
+    const BlockSigns<RB, NEG> sg(p, op, tbase, lt);
+#pragma unroll
+    for (int r = 0; r < (1 << RB); ++r) {
+        const uint32_t m = ((minus >> r) & 1u) << 31;
+        if ((NEG & (0x80u | (uint32_t)r)) == 0) {
+            if (m) a[r] = cneg<R>(a[r]);
+        } else if constexpr (sizeof(R) == 4) {
+            const float s = __uint_as_float(0x3f800000u ^ m ^ sg.at(r));
+            a[r] = pmul(a[r], make_float2(s, s));
+        } else {
+            a[r] = csign<R>(a[r], m ^ sg.at(r));
+        }
+    }
+}
+
 // per-member rotation on register bit J: RY [[c, -s], [s, c]] (real, packed
 // FMAs) or RX [[c, -i s], [-i s, c]], for the registers whose bits of mr are 1
 template <typename R, int RB, int J>
@@ -521,9 +600,11 @@ __device__ __forceinline__ void tile_tables(const TileParams<R> &p, uint32_t *ta
         ltab[s * NT + threadIdx.x] = (uint16_t)lt;
         if (s == 0) continue;
         uint32_t w = swizzle_pos<R>(thread_local_index<WB>(p.st[s - 1], lane, warp), st.fcol, p.k) * sizeof(V<R>);
+#ifndef QSIM_PASS_KERNEL
         // the previous stage's register frame: register r is written where r ^ rflip belongs
         for (int j = 0; j < RB; ++j)
             if ((p.st[s - 1].rflip >> j) & 1u) w ^= st.rw[j];
+#endif
         const uint32_t r = swizzle_pos<R>(lt, st.fcol, p.k) * sizeof(V<R>);
         tab[s * NT + threadIdx.x] = w | (r << 16);
     }
@@ -550,25 +631,46 @@ __device__ __forceinline__ void tile_load(V<R> *a, const V<R> *__restrict__ psi,
     uint64_t gr[RB];
 #pragma unroll
     for (int j = 0; j < RB; ++j) gr[j] = 1ull << p.gbit[s0.rloc[j]];
+    // (register bits are not among the thread's or the tile's: offsets add up)
+    const V<R> *src = psi + gt;
 #pragma unroll
     for (int r = 0; r < (1 << RB); ++r) {
         if constexpr (is_dd<R>) {  // complex128 in memory, split into double-float pairs
-            const double2 v = reinterpret_cast<const double2 *>(psi)[gt | reg_offset<RB>(r, gr)];
+            const double2 v = reinterpret_cast<const double2 *>(src)[reg_offset<RB>(r, gr)];
             a[r] = mkc<dd>(dd(v.x), dd(v.y));
         } else {
-            a[r] = psi[gt | reg_offset<RB>(r, gr)];
+            a[r] = src[reg_offset<RB>(r, gr)];
         }
     }
 }
 
 // Transpose into stage s (s > 0): write under the previous mapping, read under
 // this one (positions are linear over XOR: thread offset ^ register offsets).
+// In a specialised kernel the register offsets are constants, and only their
+// low (swizzled) position bits overlap the thread's: the high ones are added,
+// as the access's own constant offset, so that at most 2^h XORs are left of 32.
 template <typename R, int RB>
 __device__ __forceinline__ void tile_transpose(V<R> *a, unsigned char *smem, const uint32_t *tab,
                                                const TileParams<R> &p, int s) {
     constexpr int NT = 32 << TileCfg<R>::WB;
     const TileStage &st = p.st[s];
     const uint32_t e = tab[s * NT + threadIdx.x];
+#ifdef QSIM_PASS_KERNEL
+    constexpr uint32_t low = ((1u << swizzle_low_bits<R>()) - 1u) * (uint32_t)sizeof(V<R>);
+    auto at = [&](uint32_t thread, int r, const uint16_t *o) {
+        uint32_t off = 0;
+#pragma unroll
+        for (int j = 0; j < RB; ++j)
+            if ((r >> j) & 1) off ^= o[j];
+        return smem + (thread ^ (off & low)) + (off & ~low);
+    };
+    const int frame = p.st[s - 1].rflip;  // register r is written where r ^ frame belongs
+#pragma unroll
+    for (int r = 0; r < (1 << RB); ++r) *reinterpret_cast<V<R> *>(at(e & 0xffffu, r ^ frame, st.rw)) = a[r];
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < (1 << RB); ++r) a[r] = *reinterpret_cast<const V<R> *>(at(e >> 16, r, st.rr));
+#else
     uint32_t ro[RB];
 #pragma unroll
     for (int j = 0; j < RB; ++j) ro[j] = st.rw[j];
@@ -581,6 +683,7 @@ __device__ __forceinline__ void tile_transpose(V<R> *a, unsigned char *smem, con
 #pragma unroll
     for (int r = 0; r < (1 << RB); ++r)
         a[r] = *reinterpret_cast<const V<R> *>(smem + ((e >> 16) ^ reg_local<RB>(r, ro)));
+#endif
     __syncthreads();
 }
 
@@ -875,17 +978,20 @@ __device__ __forceinline__ void tile_store(V<R> *__restrict__ psi, const V<R> *a
         if ((warp >> w) & 1) gt |= 1ull << p.gbit[sl.wloc[w]];
     uint64_t gr[RB];
 #pragma unroll
-    for (int j = 0; j < RB; ++j) {
-        gr[j] = 1ull << p.gbit[sl.rloc[j]];
-        if ((sl.rflip >> j) & 1u) gt |= gr[j];  // register frame: r holds r ^ rflip
-    }
+    for (int j = 0; j < RB; ++j) gr[j] = 1ull << p.gbit[sl.rloc[j]];
+#ifdef QSIM_PASS_KERNEL
+    V<R> *dst = psi + gt;
+    auto at = [&](int r) { return dst + reg_offset<RB>(r ^ sl.rflip, gr); };  // register frame: r holds r ^ rflip
+#else
+    gt |= reg_offset<RB>(sl.rflip, gr);
+    auto at = [&](int r) { return psi + (gt ^ reg_offset<RB>(r, gr)); };
+#endif
 #pragma unroll
     for (int r = 0; r < (1 << RB); ++r) {
         if constexpr (is_dd<R>)
-            reinterpret_cast<double2 *>(psi)[gt ^ reg_offset<RB>(r, gr)] =
-                make_double2(to_double(re_of<dd>(a[r])), to_double(im_of<dd>(a[r])));
+            *reinterpret_cast<double2 *>(at(r)) = make_double2(to_double(re_of<dd>(a[r])), to_double(im_of<dd>(a[r])));
         else
-            psi[gt ^ reg_offset<RB>(r, gr)] = a[r];
+            *at(r) = a[r];
     }
 }
 

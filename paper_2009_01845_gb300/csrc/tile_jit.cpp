@@ -27,6 +27,7 @@
 
 #include <atomic>
 #include <chrono>
+#include <cmath>
 #include <condition_variable>
 #include <cstdarg>
 #include <cstdio>
@@ -213,6 +214,105 @@ template <typename T> int used(const T *a, int n) {
     return n;
 }
 
+// ------------------------------------------------------------------ diagonal blocks
+// The blocks of a pass that diag_table or diag_signs runs: all factors under
+// thread or outside bits are signs. `flips` uniform sign flips directly before
+// the block are folded into it. A block whose constants are all +1 or -1 is
+// signs alone (`minus`: the registers it negates); its constants stay in the
+// pass's key, the others' phases have places in the value block.
+struct DiagBlock {
+    int op = 0, flips = 0;
+    int tab = -1;        // first entry of the table, or -1: signs alone
+    uint32_t minus = 0;
+    uint32_t neg = 0;    // bits the sign factors may negate
+};
+
+// +1 or -1, with no imaginary part
+template <typename R> bool unit_sign(const V<R> &v, bool *minus) {
+    if constexpr (is_dd<R>) {
+        *minus = v.h.x < 0;
+        return std::fabs(v.h.x) == 1.f && v.l.x == 0.f && v.h.y == 0.f && v.l.y == 0.f;
+    } else {
+        *minus = v.x < 0;
+        return std::fabs(v.x) == (R)1 && v.y == (R)0;
+    }
+}
+
+template <typename R> std::vector<DiagBlock> diag_blocks(const TileParams<R> &P) {
+    constexpr int RB = TileCfg<R>::RB, NR = 1 << RB;
+    std::vector<DiagBlock> out;
+    int tables = 0;
+    for (int s = 0; s < P.n_stages; ++s) {
+        int flips = 0;
+        for (int o = P.st[s].op_begin; o < P.st[s].op_end; ++o) {
+            const TileOp &op = P.op[o];
+            if (op.type == TOP_FLIP && op.mt == 0 && op.mo == 0) {
+                ++flips;
+                continue;
+            }
+            const int f = flips;
+            flips = 0;
+            // outside factors (gl), others under thread bits, pairs (a): none
+            if (op.type != TOP_DBLOCK || op.gl != 0 || op.a != 0 || op.b != op.tkind) continue;
+            DiagBlock d;
+            d.op = o;
+            d.flips = f;
+            for (int i = 0; i < op.tkind; ++i) d.neg |= P.dfac[(int)op.mo + i].a;
+            bool signs = true, m[1 + RB];
+            for (int j = 0; j <= RB; ++j) signs = signs && unit_sign<R>(P.mat[op.m + j], &m[j]);
+            if (signs) {
+                for (int r = 0; r < NR; ++r) {
+                    bool neg = m[0];
+                    for (int j = 0; j < RB; ++j) neg ^= ((r >> j) & 1) && m[1 + j];
+                    d.minus |= (uint32_t)neg << r;
+                }
+            } else {
+                if (tables == kTileMaxTables) continue;
+                d.tab = NR * tables++;
+            }
+            out.push_back(d);
+        }
+    }
+    return out;
+}
+
+// registers that the flip op negates (dispatch_flip)
+template <typename R> uint32_t flip_mask(const TileOp &op) {
+    uint32_t m = 0;
+    const uint32_t need = op.mr | (1u << op.a) | (1u << op.b);
+    const uint32_t frame = (op.mr ? op.fx : 0u) | ((op.tkind & 1u) << op.a) | (((op.tkind >> 1) & 1u) << op.b);
+    for (uint32_t r = 0; r < (1u << TileCfg<R>::RB); ++r)
+        if (((r ^ frame) & need) == need) m |= 1u << r;
+    return m;
+}
+template <typename R> uint32_t folded_flips(const TileParams<R> &P, const DiagBlock &d) {
+    uint32_t m = 0;
+    for (int o = d.op - d.flips; o < d.op; ++o) m ^= flip_mask<R>(P.op[o]);
+    return m;
+}
+
+// the block's phases: the base times the ratios of the register's set bits,
+// multiplied in FP64 and rounded once
+template <typename R> void fill_table(const TileParams<R> &P, const DiagBlock &d, V<R> *tab) {
+    constexpr int RB = TileCfg<R>::RB;
+    auto val = [](const V<R> &v) {
+        if constexpr (is_dd<R>)
+            return cd((double)v.h.x + (double)v.l.x, (double)v.h.y + (double)v.l.y);
+        else
+            return cd(v.x, v.y);
+    };
+    const V<R> *C = &P.mat[P.op[d.op].m];
+    const uint32_t minus = folded_flips<R>(P, d);
+    cd ph[1 << RB];
+    ph[0] = val(C[0]);
+    for (int j = 0; j < RB; ++j)
+        for (int r = 0; r < (1 << j); ++r) ph[r | (1 << j)] = ph[r] * val(C[1 + j]);
+    for (int r = 0; r < (1 << RB); ++r) {
+        const cd v = ((minus >> r) & 1u) ? -ph[r] : ph[r];
+        tab[d.tab + r] = mkc<R>(R(v.real()), R(v.imag()));
+    }
+}
+
 // folded: the pass's values are compiled in too (kP holds them); otherwise
 // they come from the value block v at run time
 template <typename R> std::string generate(const TileParams<R> &P, bool folded) {
@@ -277,6 +377,22 @@ template <typename R> std::string generate(const TileParams<R> &P, bool folded) 
         o.s += (i % 4 == 3) ? ",\n" : ",";
     }
     o.s += "}};\n\n";
+    const std::vector<DiagBlock> blocks = diag_blocks<R>(P);
+    if (folded) {
+        std::vector<V<R>> tab((size_t)kTileMaxTables << RB);
+        int n = 1;
+        for (const DiagBlock &d : blocks) {
+            if (d.tab < 0) continue;
+            fill_table<R>(P, d, tab.data());
+            n = d.tab + (1 << RB);
+        }
+        o.f("__device__ constexpr V<%s> kTab[%d] = {\n", RT, n);
+        for (int i = 0; i < n; ++i) {
+            cplx_lit<R>(o, tab[i]);
+            o.s += (i % 4 == 3) ? ",\n" : ",";
+        }
+        o.s += "};\n\n";
+    }
     // the kernel: the generic kernel's loop over stages and ops, unrolled here
     const int NT = 32 << WB;
     o.f("extern \"C\" __global__ void __launch_bounds__(%d, %d) qs_tile_pass(V<%s> *__restrict__ psi,\n"
@@ -303,9 +419,22 @@ template <typename R> std::string generate(const TileParams<R> &P, bool folded) 
         o.s += "    {\n";
         if (st.need_lt) o.f("      const uint32_t lt = ltab[%d * (NW * 32) + threadIdx.x];\n", s);
         else o.s += "      const uint32_t lt = 0u;\n";
-        for (int op = st.op_begin; op < st.op_end; ++op)
-            o.f("      tile_op<R, RB, 2>(a, kP, %s, q, %d, kP.st[%d], t, tbase, lt, lane, warp, sc);\n",
-                folded ? "kP.mat, kP.dfac" : "v.mat, v.dfac", op, s);
+        for (int op = st.op_begin; op < st.op_end; ++op) {
+            // a block with its flips, or the flips before one
+            const DiagBlock *d = nullptr;
+            for (const DiagBlock &b : blocks)
+                if (b.op - b.flips <= op && op <= b.op) d = &b;
+            if (!d) {
+                o.f("      tile_op<R, RB, 2>(a, kP, %s, q, %d, kP.st[%d], t, tbase, lt, lane, warp, sc);\n",
+                    folded ? "kP.mat, kP.dfac" : "v.mat, v.dfac", op, s);
+            } else if (op == d->op && d->tab >= 0) {
+                o.f("      diag_table<R, RB, %uu>(a, kP, %s + %d, kP.op[%d], tbase, lt);\n", d->neg,
+                    folded ? "kTab" : "v.tab", d->tab, op);
+            } else if (op == d->op) {
+                o.f("      diag_signs<R, RB, %uu>(a, kP, %uu, kP.op[%d], tbase, lt);\n", d->neg,
+                    d->minus ^ folded_flips<R>(P, *d), op);
+            }
+        }
         o.s += "    }\n";
     }
     o.s += "    tile_store<R, RB>(psi, a, kP, tbase, lane, warp);\n";
@@ -480,8 +609,9 @@ qs_status tile_jit_launch_t(qs_state *s, const TileParams<R> &p, bool *launched)
     // keys: flags (kTypeCode, kKeyFolded: values compiled in), then the
     // descriptor with its run-time pointers and the Ising op's tau (which only
     // the table kernel reads) cleared; the structure key also clears the
-    // values (matrix entries, diagonal factors)
+    // values (matrix entries, diagonal factors) but for signs
     static thread_local std::vector<unsigned char> full, key;  // reused between launches
+    const std::vector<DiagBlock> blocks = diag_blocks<R>(p);
     const size_t bytes = 1 + sizeof(TileParams<R>);
     auto fill = [&](std::vector<unsigned char> &dst, unsigned char flags) {
         dst.resize(bytes);
@@ -499,6 +629,10 @@ qs_status tile_jit_launch_t(qs_state *s, const TileParams<R> &p, bool *launched)
             if (p.op[o].type == TOP_ISING) clear(&p.op[o].tmask, sizeof(p.op[o].tmask));
         if (flags & kKeyFolded) return;
         clear(p.mat, sizeof(p.mat));
+        for (const DiagBlock &d : blocks)  // blocks of signs alone are structure
+            if (d.tab < 0)
+                std::memcpy(k + ((const unsigned char *)&p.mat[p.op[d.op].m] - (const unsigned char *)&p),
+                            &p.mat[p.op[d.op].m], (1 + TileCfg<R>::RB) * sizeof(V<R>));
         for (int f = 0; f < kTileMaxDFac; ++f) {
             clear(&p.dfac[f].v0, sizeof(p.dfac[f].v0));
             clear(&p.dfac[f].v1, sizeof(p.dfac[f].v1));
@@ -622,6 +756,8 @@ qs_status tile_jit_launch_t(qs_state *s, const TileParams<R> &p, bool *launched)
     TileVals<R> &vals = *reinterpret_cast<TileVals<R> *>(vals_buf<R>());
     std::memcpy(vals.mat, p.mat, sizeof(vals.mat));
     std::memcpy(vals.dfac, p.dfac, sizeof(vals.dfac));
+    for (const DiagBlock &d : blocks)
+        if (d.tab >= 0) fill_table<R>(p, d, vals.tab);
     void *args[] = {&psi, &q, &vals};
     QS_CUDA_TRY(cudaLaunchKernel((const void *)e->kern, dim3((unsigned)grid), dim3(32 << TileCfg<R>::WB), args,
                                  e->smem, s->stream));

@@ -209,10 +209,14 @@ template <typename R> struct TilePtrs {
 // The values of a pass (matrix entries, diagonal-block factors), passed
 // beside a specialised kernel whose descriptor holds only the structure: one
 // kernel serves every pass of that structure (e.g. every step of a Trotter
-// evolution, whose angles change from step to step).
+// evolution, whose angles change from step to step). tab: the phases of the
+// diagonal blocks that are the same in every thread up to signs, one per
+// register, formed on the host (see diag_table).
+constexpr int kTileMaxTables = 24;
 template <typename R> struct TileVals {
     V<R> mat[kTileMaxMat];
     TileDFac<R> dfac[kTileMaxDFac];  // only v0, v1, v2 are read
+    V<R> tab[kTileMaxTables << TileCfg<R>::RB];
 };
 static_assert(sizeof(TileVals<double>) <= 24576, "pass values exceed the kernel parameter budget");
 
