@@ -450,16 +450,35 @@ static qs_status emit_and_run(qs_state *s, const std::vector<LGate> &G, const st
         }
         return r;
     };
-    // lanes: the 5 lowest bits that are not registers (ops never act on lane
-    // bits; keeping index bits 0 and 1 on lanes lets the last stage store whole
-    // 32-byte sectors from any lane map), ordered, where possible, so that the
-    // lanes of a half-warp (complex64) / quarter-warp (complex128) have
-    // distinct residues, which the default swizzle then serves
+    // Warp bits of a new stage with register set rset, opened at entry `from`. A
+    // transpose that leaves the warp bits as they are moves amplitudes inside
+    // warps only and needs no CTA barrier (tile_jit.cpp), so they stay while no
+    // register takes one; else the bits needed last become the warp bits, none
+    // of the low ones (a swizzle mixes those into every position) and, in a last
+    // stage, the highest (lanes on low bits store whole lines). Lanes: the rest
+    // (ops never act on lane bits; index bits 0 and 1 on lanes let the last stage
+    // store whole 32-byte sectors), ordered, where possible, so that the lanes of
+    // a half-warp (complex64) / quarter-warp (complex128) have distinct residues,
+    // which the default swizzle then serves.
     const int half = sizeof(R) == 4 ? 4 : 3;
-    auto lanes_for = [&](int, uint32_t rset) {
+    const uint32_t all_local = (1u << k) - 1u;
+    auto warps_for = [&](int from, uint32_t rset, uint32_t prev) {
+        if ((prev & rset) == 0 && (prev & ((1u << half) - 1u)) == 0) return prev;
+        bool last = true;
+        for (int lb = 0; lb < k; ++lb)
+            if (!((rset >> lb) & 1u) && next_use[(size_t)from * k + lb] != std::numeric_limits<int>::max()) last = false;
+        std::vector<std::pair<int, int>> rank;  // (next use, local bit), furthest first
+        for (int lb = half; lb < k; ++lb)
+            if (!((rset >> lb) & 1u)) rank.push_back({last ? 0 : -next_use[(size_t)from * k + lb], -lb});
+        std::sort(rank.begin(), rank.end());
+        uint32_t w = 0;
+        for (int i = 0; i < TileCfg<R>::WB; ++i) w |= 1u << -rank[i].second;
+        return w;
+    };
+    auto lanes_for = [&](uint32_t rset, uint32_t wset) {
         std::vector<int> L;
-        for (int lb = 0; lb < k && (int)L.size() < kTileLaneBits; ++lb)
-            if (!((rset >> lb) & 1u)) L.push_back(lb);
+        for (int lb = 0; lb < k; ++lb)
+            if (!(((rset | wset) >> lb) & 1u)) L.push_back(lb);
         std::vector<int> best = L;
         do {
             bool okr = true;
@@ -481,13 +500,13 @@ static qs_status emit_and_run(qs_state *s, const std::vector<LGate> &G, const st
     // entries with and without them (capacity is not checked here).
     if (count_only) {
         uint32_t c = choose(0, (ne ? needl[0] : 0u) & high_bits, high_bits);
-        uint32_t lanes = low5_mask;
+        uint32_t lanes = low5_mask, wset = all_local & ~c & ~lanes;
         int stages = 1;
         for (int i = 0; i < ne; ++i) {
             if ((needl[i] & ~c) == 0) continue;
             c = choose(i, needl[i], (1u << k) - 1u);
-            lanes = 0;
-            for (int lb : lanes_for(i, c)) lanes |= 1u << lb;
+            wset = warps_for(i, c, wset);
+            lanes = all_local & ~c & ~wset;
             ++stages;
         }
         const uint32_t sector_bits = sizeof(R) == 4 ? 3u : 1u;
@@ -785,7 +804,7 @@ static qs_status emit_and_run(qs_state *s, const std::vector<LGate> &G, const st
             if (nst >= kTileMaxStages) return overflow();
             if (free_lanes) {
                 const uint32_t rset = choose(oi, needl[oi], (1u << k) - 1u);
-                open_stage(rset, lanes_for(oi, rset));
+                open_stage(rset, lanes_for(rset, warps_for(oi, rset, all_local & ~cur & ~curL)));
             } else {
                 open_stage(choose(oi, needl[oi], highmask), natural);
             }

@@ -649,7 +649,11 @@ __device__ __forceinline__ void tile_load(V<R> *a, const V<R> *__restrict__ psi,
 // In a specialised kernel the register offsets are constants, and only their
 // low (swizzled) position bits overlap the thread's: the high ones are added,
 // as the access's own constant offset, so that at most 2^h XORs are left of 32.
-template <typename R, int RB>
+// LOCAL: both stages have the same warp bits, none of them among the swizzled
+// low ones: a warp writes and reads positions of its own, and the warps need not
+// meet. BEFORE: other warps may still be reading for an earlier local transpose
+// whose positions are not this warp's now: they meet first.
+template <typename R, int RB, bool LOCAL = false, bool BEFORE = false>
 __device__ __forceinline__ void tile_transpose(V<R> *a, unsigned char *smem, const uint32_t *tab,
                                                const TileParams<R> &p, int s) {
     constexpr int NT = 32 << TileCfg<R>::WB;
@@ -664,12 +668,18 @@ __device__ __forceinline__ void tile_transpose(V<R> *a, unsigned char *smem, con
             if ((r >> j) & 1) off ^= o[j];
         return smem + (thread ^ (off & low)) + (off & ~low);
     };
+    auto meet = [] {
+        if (LOCAL) __syncwarp();
+        else __syncthreads();
+    };
     const int frame = p.st[s - 1].rflip;  // register r is written where r ^ frame belongs
+    if (BEFORE) __syncthreads();
 #pragma unroll
     for (int r = 0; r < (1 << RB); ++r) *reinterpret_cast<V<R> *>(at(e & 0xffffu, r ^ frame, st.rw)) = a[r];
-    __syncthreads();
+    meet();
 #pragma unroll
     for (int r = 0; r < (1 << RB); ++r) a[r] = *reinterpret_cast<const V<R> *>(at(e >> 16, r, st.rr));
+    meet();
 #else
     uint32_t ro[RB];
 #pragma unroll
@@ -683,8 +693,8 @@ __device__ __forceinline__ void tile_transpose(V<R> *a, unsigned char *smem, con
 #pragma unroll
     for (int r = 0; r < (1 << RB); ++r)
         a[r] = *reinterpret_cast<const V<R> *>(smem + ((e >> 16) ^ reg_local<RB>(r, ro)));
-#endif
     __syncthreads();
+#endif
 }
 
 // Per-warp gradient sums: in the state's precision, double for double-float.

@@ -313,6 +313,37 @@ template <typename R> void fill_table(const TileParams<R> &P, const DiagBlock &d
     }
 }
 
+// How the transpose into each stage synchronises. A transpose between stages
+// with the same warp bits, none of them among the swizzled low position bits,
+// stays inside each warp's own positions (the swizzle maps the positions with
+// given warp bits to themselves). A transpose that is not local, or is local in
+// other positions, waits for the CTA first if a local one came before it: in the
+// loop over tiles the pass's last transpose comes before its first. (The FMA
+// pipe and shared memory take turns where a CTA's warps move together: a stage
+// took their sum, 2400 cycles a tile, with 2 CTAs per SM. Random layers n = 28
+// complex64, 27 of 83 transposes local: 25.0 -> 24.5 ms; energy and gradient at
+// n = 18, 64 members 3.08 -> 2.98 ms. Tiles of 2^12 in CTAs of 4 warps, 4 per SM,
+// run a pass 13% faster but need 13 passes for 11: 25.5 ms.)
+constexpr char kSyncLocal = 1, kSyncBefore = 2;
+template <typename R> std::vector<char> transpose_sync(const TileParams<R> &P) {
+    constexpr int WB = TileCfg<R>::WB;
+    std::vector<char> out(P.n_stages, 0);
+    auto warps = [&](int s) {
+        int w = 0;
+        for (int i = 0; i < WB; ++i) w |= 1 << P.st[s].wloc[i];
+        return w;
+    };
+    int open = 0;  // warp bits of the local transposes since the CTA last met (0: none)
+    for (int round = 0; round < 2; ++round)
+        for (int s = 1; s < P.n_stages; ++s) {
+            const int w = warps(s);
+            const bool local = w == warps(s - 1) && (w & ((1 << swizzle_low_bits<R>()) - 1)) == 0;
+            out[s] = (local ? kSyncLocal : 0) | (open != 0 && !(local && open == w) ? kSyncBefore : 0);
+            open = local ? w : 0;
+        }
+    return out;
+}
+
 // folded: the pass's values are compiled in too (kP holds them); otherwise
 // they come from the value block v at run time
 template <typename R> std::string generate(const TileParams<R> &P, bool folded) {
@@ -413,9 +444,12 @@ template <typename R> std::string generate(const TileParams<R> &P, bool folded) 
         "  for (uint64_t t = blockIdx.x; t < kP.total_tiles; t += gridDim.x) {\n"
         "    const uint64_t tbase = tile_base<R>(kP, t);\n"
         "    tile_load<R, RB>(a, psi, kP, tbase, lane, warp);\n";
+    const std::vector<char> sync = transpose_sync<R>(P);
     for (int s = 0; s < P.n_stages; ++s) {
         const TileStage &st = P.st[s];
-        if (s > 0) o.f("    tile_transpose<R, RB>(a, smem_raw, tab, kP, %d);\n", s);
+        if (s > 0)
+            o.f("    tile_transpose<R, RB, %s, %s>(a, smem_raw, tab, kP, %d);\n", (sync[s] & kSyncLocal) ? "true" : "false",
+                (sync[s] & kSyncBefore) ? "true" : "false", s);
         o.s += "    {\n";
         if (st.need_lt) o.f("      const uint32_t lt = ltab[%d * (NW * 32) + threadIdx.x];\n", s);
         else o.s += "      const uint32_t lt = 0u;\n";
