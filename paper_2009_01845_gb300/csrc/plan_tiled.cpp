@@ -6,8 +6,8 @@
 //     gates need no tile bits at all, since a tile knows every index bit of
 //     every amplitude it holds.
 // A gate the tile cannot express (dense on 3+ qubits, a general 2+-qubit
-// diagonal, for complex128 a SWAP of a lane bit) is applied by its own unfused
-// pass when it reaches the front of the queue. Within a pass, stages re-split
+// diagonal, in double-float a 2-qubit gate of a lane bit) is applied by its own
+// unfused pass when it reaches the front of the queue. Within a pass, stages re-split
 // the tile's bits, lane bits included, between registers, lanes and warps; the
 // register set of a new stage is the needed bits plus the bits used soonest
 // afterwards (furthest-next-use eviction).
@@ -34,9 +34,11 @@ namespace {
 
 enum GClass { G_PHASE, G_DIAG1, G_DENSE1, G_DENSE2, G_SWAP, G_GRAD, G_ISING, G_SINGLE };
 
-// low_swaps: SWAPs that touch a lane bit may run in a tile too (complex128 in
-// double-float keeps those in passes of their own, which move amplitudes exactly)
-GClass classify(const LGate &g, bool low_swaps) {
+// low_pairs: 2-qubit gates and SWAPs that touch a lane bit may run in a tile too.
+// Complex128 in double-float keeps those in passes of their own: one-gate SWAPs
+// move amplitudes exactly, and a double-float 4x4 gate makes a specialised pass
+// slow to compile (2 of them 14 s, 4 of them 47 s).
+GClass classify(const LGate &g, bool low_pairs) {
     if (g.kind == kKindGrad) return G_GRAD;
     if (g.kind == kKindIsing) return G_ISING;
     if (g.param_index >= 0) {
@@ -50,11 +52,10 @@ GClass classify(const LGate &g, bool low_swaps) {
     }
     if (g.phase_only) return G_PHASE;
     if (g.diagonal) return g.k == 1 ? G_DIAG1 : G_SINGLE;
-    if (g.is_swap)
-        return low_swaps || (g.tbit[0] >= kTileLaneBits && g.tbit[1] >= kTileLaneBits) ? G_SWAP : G_SINGLE;
+    const bool pair = g.k == 2 && (low_pairs || (g.tbit[0] >= kTileLaneBits && g.tbit[1] >= kTileLaneBits));
+    if (g.is_swap) return pair ? G_SWAP : G_SINGLE;
     if (g.k == 1) return G_DENSE1;
-    if (g.k == 2) return G_DENSE2;
-    return G_SINGLE;
+    return pair ? G_DENSE2 : G_SINGLE;
 }
 
 uint64_t qubit_bits(const LGate &g) {
@@ -1405,8 +1406,8 @@ qs_status run_tiled(qs_state *s, const std::vector<LGate> &G, const double *para
     const int nh = k - kTileLaneBits;  // chosen high tile bits
     const uint64_t force = force_bit >= 0 ? (1ull << force_bit) : 0ull;
     std::vector<GClass> cls(G.size());
-    const bool low_swaps = s->dtype == QS_C64 || c128_fp64();
-    for (size_t i = 0; i < G.size(); ++i) cls[i] = classify(G[i], low_swaps);
+    const bool low_pairs = s->dtype == QS_C64 || c128_fp64();
+    for (size_t i = 0; i < G.size(); ++i) cls[i] = classify(G[i], low_pairs);
     // per-member matrices of every batched-parameter gate, built once on the device
     std::vector<int> slot(G.size(), -1), spidx, skind;
     for (size_t i = 0; i < G.size(); ++i)
