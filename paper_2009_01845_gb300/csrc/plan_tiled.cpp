@@ -74,6 +74,10 @@ uint64_t target_bits(const LGate &g, GClass c) {
 // the high (non-lane) ones: the tile has to include them
 uint64_t need_bits(const LGate &g, GClass c) { return target_bits(g, c) & ~((1ull << kTileLaneBits) - 1ull); }
 
+// 2-qubit gates of lane bits in one pass: a specialised pass with 16 of them
+// takes 5.5 s to compile, and the time grows faster than their number
+constexpr int kMaxLowPairs = 16;
+
 int mat_entries(GClass c) {
     switch (c) {
     case G_PHASE: return 1;
@@ -1435,6 +1439,7 @@ qs_status run_tiled(qs_state *s, const std::vector<LGate> &G, const double *para
             out->high = force | fixed_high;
             out->gates.clear();
             uint64_t blocked = 0;
+            int low2 = 0;
             for (size_t i = first; i < G.size(); ++i) {
                 if (done[i]) continue;
                 if (blocked == all_bits) break;  // nothing later can join this pass
@@ -1449,6 +1454,10 @@ qs_status run_tiled(qs_state *s, const std::vector<LGate> &G, const double *para
                 }
                 const uint64_t nb = need_bits(G[i], cls[i]);
                 if (fixed ? (nb & ~out->high) != 0 : __builtin_popcountll(out->high | nb) > nh) {
+                    blocked |= qb;
+                    continue;
+                }
+                if (cls[i] == G_DENSE2 && (qb & ((1ull << kTileLaneBits) - 1ull)) && ++low2 > kMaxLowPairs) {
                     blocked |= qb;
                     continue;
                 }
