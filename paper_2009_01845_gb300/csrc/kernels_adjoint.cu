@@ -117,12 +117,35 @@ __global__ void __launch_bounds__(256) grad_reduce_kernel(const double *__restri
     if (threadIdx.x == 0) grad[(uint64_t)b * p.n_params + p.param0 + pi] = total;
 }
 
+// The same with a warp per row: up to kWarpTiles tiles per member a CTA per row
+// leaves most of its threads without a tile (n = 18, 64 members, 180 rows of 64
+// tiles: 49 us; energy and gradient 2.98 -> 2.95 ms).
+constexpr uint64_t kWarpTiles = 256;
+
+__global__ void __launch_bounds__(256) grad_reduce_warp_kernel(const double *__restrict__ part,
+                                                               const __grid_constant__ GradReduceP p, int rows,
+                                                               double *__restrict__ grad) {
+    const int pi = blockIdx.x * 8 + (threadIdx.x >> 5), b = blockIdx.y, lane = threadIdx.x & 31;
+    if (pi >= rows) return;
+    double total = 0.0;
+    for (int k = p.beg[pi]; k < p.beg[pi + 1]; ++k) {
+        const double *row = part + (uint64_t)p.slot[k] * p.total_tiles + (uint64_t)b * p.tiles_per_member;
+        double acc = 0.0;
+        for (uint64_t t = lane; t < p.tiles_per_member; t += 32) acc += row[t];
+        for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
+        total += p.coef[k] * acc;
+    }
+    if (lane == 0) grad[(uint64_t)b * p.n_params + p.param0 + pi] = total;
+}
+
 qs_status k_grad_reduce(const double *part, const GradReduceP &p, int n_param_rows, int batch, double *grad,
                         cudaStream_t st) {
     if (n_param_rows <= 0) return QS_OK;
     ProfScope _ps(st, KC_ADJOINT);
-    dim3 grid(n_param_rows, batch);
-    grad_reduce_kernel<<<grid, 256, 0, st>>>(part, p, grad);
+    if (p.tiles_per_member <= kWarpTiles)
+        grad_reduce_warp_kernel<<<dim3((n_param_rows + 7) / 8, batch), 256, 0, st>>>(part, p, n_param_rows, grad);
+    else
+        grad_reduce_kernel<<<dim3(n_param_rows, batch), 256, 0, st>>>(part, p, grad);
     QS_CUDA_TRY(cudaGetLastError());
     return QS_OK;
 }

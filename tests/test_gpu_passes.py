@@ -24,9 +24,11 @@ def qs():
     qsim.jit_set_policy("tiered")
 
 
-def low_two_qubit(n, r):
+# complex128 circuits are short: a specialised double-float pass takes seconds
+# to compile, one with 4x4 gates far longer
+def low_two_qubit(n, r, long):
     g = []
-    for k in range(40):
+    for k in range(12 if long else 3):
         a, b = (int(x) for x in r.permutation(6)[:2])          # index bits 0 .. 5
         q = (n - 1 - a, n - 1 - b)
         g.append(qi.Gate("SWAP", q) if k % 3 == 0 else qi.Gate("UNITARY", q, (), (), qi.random_unitary(2, r)))
@@ -36,9 +38,9 @@ def low_two_qubit(n, r):
     return g
 
 
-def diagonals(n, r):
+def diagonals(n, r, long):
     g = []
-    for layer in range(8):
+    for layer in range(8 if long else 2):
         for q in range(n):
             if layer % 2:
                 g.append(qi.Gate("RY", (q,), (), (float(r.uniform(0, 6.28)),)))
@@ -54,14 +56,21 @@ def diagonals(n, r):
 
 
 @pytest.mark.parametrize("policy", ["off", "sync"])
-@pytest.mark.parametrize("dtype,n", [("c64", 13), ("c64", 15), ("c128", 12), ("c128", 15)])
+@pytest.mark.parametrize("dtype,n,fp64", [("c64", 13, False), ("c64", 15, False), ("c128", 12, False),
+                                          ("c128", 15, False), ("c128", 13, True)])
 @pytest.mark.parametrize("circuit", [low_two_qubit, diagonals])
-def test_pass_kernels(qs, circuit, dtype, n, policy):
-    gates = circuit(n, qi.rng(17 * n))
+def test_pass_kernels(qs, circuit, dtype, n, fp64, policy):
+    gates = circuit(n, qi.rng(17 * n), dtype == "c64")
     psi = qi.random_state(n, n)
     want = oracle.apply_circuit(psi.copy(), n, gates)
     qs.jit_set_policy(policy)
-    got = qs.State(n, dtype=dtype).set(psi).apply(gates, mode="tiled").get()
+    before = qs.jit_stats()
+    got = qs.State(n, dtype=dtype).set(psi).apply(gates, mode="tiled", fp64=fp64).get()
+    after = qs.jit_stats()
+    assert after["failed"] == before["failed"]
+    if policy == "sync":  # every pass ran on its specialised kernel
+        assert after["generic_launches"] == before["generic_launches"]
+        assert after["specialised_launches"] > before["specialised_launches"]
     mx, l2 = TOL[dtype]
     assert np.max(np.abs(got - want)) <= mx and np.linalg.norm(got - want) <= l2
 
@@ -73,3 +82,24 @@ def test_low_swaps_of_complex128_are_exact(qs, n):
     want = oracle.apply_circuit(psi.copy(), n, gates)
     got = qs.State(n, dtype="c128").set(psi).apply(gates).get()
     np.testing.assert_array_equal(got, want)
+
+
+@pytest.mark.parametrize("n", [13, 20, 21])
+def test_gradient_over_few_and_many_tiles(qs, n):
+    """2, 256 and 512 tiles per member (complex64): the reduction's two forms,
+    against parameter shifts of the energy (tolerance: the energies' rounding,
+    2^-24 per gate on amplitudes, 2 sum|c|)."""
+    import torch
+    gates = qi.variational_circuit(n, np.zeros((2, n)))
+    index, count = qs.param_indices(gates)
+    terms = qi.tfim_terms(n, 0.9)
+    eng = qs.EnergyGradient(n, 1, gates, index, terms)
+    params = torch.from_numpy(qi.rng(n).uniform(0, 6.28, size=(1, count))).cuda()
+    grad = eng.run(params)[1].cpu().numpy().copy()
+    for j in (0, 7, 8, n, count - 1):
+        e = []
+        for sign in (1.0, -1.0):
+            p = params.clone()
+            p[:, j] += sign * np.pi / 2
+            e.append(float(eng.run(p, mode="forward")[0].cpu()))
+        assert abs((e[0] - e[1]) / 2 - grad[0, j]) <= 2 * sum(abs(t[0]) for t in terms) * len(gates) * 2.0 ** -24
