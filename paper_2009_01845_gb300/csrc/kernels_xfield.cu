@@ -12,12 +12,17 @@
 // no bank conflicts). The first pass has the 12 lowest index bits in the tile;
 // a later pass has the 4 lowest (whole 128-byte lines of complex64) and a
 // window of 8 others: 12 + 8 per further pass, so 3 reads of the state for 27
-// qubits instead of 27. Measured at n = 27, complex64 (1 GiB): 0.18 ms per pass
-// (0.86 of the HBM peak), 0.55 ms for the field; one launch per term, 4.8 ms.
+// qubits instead of 27. Measured at n = 27, complex64 (1 GiB): 0.19 ms per pass
+// (0.81 of the HBM peak), 0.59 ms for the field; one launch per term, 4.8 ms.
 //
-// Per thread the 16 products of a term are summed in the state's precision and
-// added to a running sum: for complex64 a float-float pair (Knuth's two-sum),
-// so nothing is lost over the tiles a thread takes; FP64 across threads.
+// Per thread the 16 products of a term are summed in the state's precision (8
+// at a time) and added to a running sum that keeps what FP64 would: complex64
+// sums the terms of 8 tiles exactly, as three floats (Knuth's two-sum twice),
+// and adds those to an FP64 sum; an FP64 addition per term would take as long
+// as the read of the state (2 per clock and SM), and a pair of floats (0.56 ms
+// at n = 27) holds 48 bits where FP64 holds 53. FP64 across threads. A state of
+// one tile (n = 12) has its complex64 products added in FP64 one by one, as
+// expect_partial_kernel does there: 26 us, 14 us in lumps of 16 products.
 #include <algorithm>
 #include <cstring>
 
@@ -47,38 +52,73 @@ template <typename R> struct XFieldP {
 template <typename R> struct RunningSum {
     R s = 0;
     __device__ __forceinline__ void add(R v) { s += v; }
+    __device__ __forceinline__ void flush() {}
     __device__ __forceinline__ double value() const { return (double)s; }
 };
 template <> struct RunningSum<float> {
-    float hi = 0.f, lo = 0.f;
-    __device__ __forceinline__ void add(float v) {
-        const float t = hi + v;
-        const float bv = t - hi;
-        lo += (hi - (t - bv)) + (v - bv);
-        hi = t;
+    double sum = 0.0;
+    float2 a = {0.f, 0.f}, b = {0.f, 0.f}, c = {0.f, 0.f};  // a + b + c, both lanes: the terms since the last flush
+    __device__ __forceinline__ static float2 two_sum(float2 &s, float2 v) {
+        const float2 t = padd(s, v), bv = psub(t, s);
+        const float2 e = padd(psub(s, psub(t, bv)), psub(v, bv));
+        s = t;
+        return e;
     }
-    __device__ __forceinline__ double value() const { return (double)hi + (double)lo; }
+    // the four terms of a view (0 where there is none)
+    __device__ __forceinline__ void add(const float *v) {
+        float2 na = a, nb = b, nc = c;
+#pragma unroll
+        for (int j = 0; j < 4; j += 2) {
+            const float2 e = two_sum(na, make_float2(v[j], v[j + 1]));
+            nc = padd(nc, two_sum(nb, e));
+        }
+        if (fabsf(na.x) + fabsf(na.y) <= 3.402823466e38f) {
+            a = na;
+            b = nb;
+            c = nc;
+        } else {  // near the end of the floats' range, infinite or NaN: FP64's result
+            flush();
+            for (int j = 0; j < 4; ++j) sum += (double)v[j];
+        }
+    }
+    __device__ __forceinline__ void flush() {
+        sum += (double)a.x + ((double)b.x + (double)c.x);
+        sum += (double)a.y + ((double)b.y + (double)c.y);
+        a = b = c = make_float2(0.f, 0.f);
+    }
+    __device__ __forceinline__ double value() const { return sum; }
 };
 
 // the terms on the 4 register bits of a[], which are tile bits b0 .. b0+3
-template <typename R>
+template <typename R, bool WIDE>
 __device__ __forceinline__ void view_terms(const V<R> *a, const XFieldP<R> &p, int b0, RunningSum<R> &acc) {
+    R v[4];
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
+        v[j] = 0;
         if (!((p.active >> (b0 + j)) & 1u)) continue;
-        R s0 = 0, s1 = 0;
+        const R c = p.c[b0 + j];
+        V<R> s = mkc<R>(0, 0);  // products of the real and of the imaginary parts
 #pragma unroll
         for (int r = 0; r < kPer; ++r) {
             if (r & (1 << j)) continue;
             const V<R> x = a[r], y = a[r | (1 << j)];
-            s0 = fma(x.x, y.x, s0);
-            s1 = fma(x.y, y.y, s1);
+            if constexpr (WIDE) {
+                acc.sum += (double)(c * fma(x.x, y.x, x.y * y.y));
+            } else if constexpr (sizeof(R) == 4) {
+                s = pfma(x, y, s);
+            } else {
+                s.x = fma(x.x, y.x, s.x);
+                s.y = fma(x.y, y.y, s.y);
+            }
         }
-        acc.add(p.c[b0 + j] * (s0 + s1));
+        if constexpr (sizeof(R) == 4) v[j] = __fmul_rn(c, s.x + s.y);  // rounded: not fused into add()'s sums
+        else acc.add(c * (s.x + s.y));
     }
+    if constexpr (sizeof(R) == 4 && !WIDE) acc.add(v);
 }
 
-template <typename R>
+template <typename R, bool WIDE>
 __global__ void __launch_bounds__(kThreads, sizeof(R) == 4 ? 4 : 2)
     expect_xfield_kernel(const V<R> *__restrict__ psi, const __grid_constant__ XFieldP<R> p,
                          double2 *__restrict__ part) {
@@ -93,13 +133,14 @@ __global__ void __launch_bounds__(kThreads, sizeof(R) == 4 ? 4 : 2)
     const uint64_t toff = (uint64_t)(tid & lom) | ((uint64_t)(tid >> (p.lo < 8 ? p.lo : 8)) << p.w);
     const int cshift = p.lo >= 8 ? 8 : 8 - p.lo + p.w;
     RunningSum<R> acc;
+    int tiles = 0;
     for (uint64_t t = blockIdx.x; t < p.tiles; t += gridDim.x) {
         const uint64_t base = ((t & ((1ull << gap) - 1ull)) << p.lo) | ((t >> gap) << (p.w + kBits - p.lo));
         const V<R> *src = q + (base | toff);
         V<R> a[kPer];
 #pragma unroll
         for (int c = 0; c < kPer; ++c) a[c] = src[(uint64_t)c << cshift];
-        if (p.active & 0xf00u) view_terms<R>(a, p, 8, acc);
+        if (p.active & 0xf00u) view_terms<R, WIDE>(a, p, 8, acc);
         if (p.active & 0x0ffu) {
             __syncthreads();  // the previous tile's readers are done
             // tile-local index l at position l ^ (bits 4..7 of l): both reads
@@ -111,16 +152,18 @@ __global__ void __launch_bounds__(kThreads, sizeof(R) == 4 ? 4 : 2)
                 const uint32_t row = (tid >> 4) << 8, col = tid & 15u;
 #pragma unroll
                 for (int c = 0; c < kPer; ++c) a[c] = tile[row | (c << 4) | (col ^ (uint32_t)c)];
-                view_terms<R>(a, p, 4, acc);
+                view_terms<R, WIDE>(a, p, 4, acc);
             }
             if (p.active & 0x00fu) {
                 const uint32_t row = tid << 4, col = tid & 15u;
 #pragma unroll
                 for (int c = 0; c < kPer; ++c) a[c] = tile[row | ((uint32_t)c ^ col)];
-                view_terms<R>(a, p, 0, acc);
+                view_terms<R, WIDE>(a, p, 0, acc);
             }
         }
+        if ((++tiles & 7) == 0) acc.flush();
     }
+    acc.flush();
     double d = acc.value();
     for (int o = 16; o > 0; o >>= 1) d += __shfl_down_sync(0xffffffffu, d, o);
     if ((tid & 31u) == 0) sh[tid >> 5] = d;
@@ -141,7 +184,7 @@ qs_status xfield_t(const V<R> *psi, int n, int ms, int batch, const double *coef
                    bool accumulate, cudaStream_t st) {
     constexpr size_t smem = sizeof(V<R>) << kBits;
     if (smem > 48 * 1024)
-        QS_CUDA_TRY(cudaFuncSetAttribute(expect_xfield_kernel<R>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        QS_CUDA_TRY(cudaFuncSetAttribute(expect_xfield_kernel<R, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)smem));
     uint64_t left = 0;  // index bits with a term not yet done
     for (int b = 0; b < n; ++b)
@@ -167,7 +210,14 @@ qs_status xfield_t(const V<R> *psi, int n, int ms, int batch, const double *coef
             const double amps = (double)((uint64_t)batch << n);
             prof_add_work(KC_REDUCE, amps * sizeof(V<R>), 2.0 * amps * __builtin_popcount(p.active));
         }
-        expect_xfield_kernel<R><<<dim3(blocks, batch), kThreads, smem, st>>>(psi, p, part);
+        if constexpr (sizeof(R) == 4) {
+            if (n == kBits)
+                expect_xfield_kernel<R, true><<<dim3(blocks, batch), kThreads, smem, st>>>(psi, p, part);
+            else
+                expect_xfield_kernel<R, false><<<dim3(blocks, batch), kThreads, smem, st>>>(psi, p, part);
+        } else {
+            expect_xfield_kernel<R, false><<<dim3(blocks, batch), kThreads, smem, st>>>(psi, p, part);
+        }
         QS_CUDA_TRY(cudaGetLastError());
     }
     return QS_OK;
