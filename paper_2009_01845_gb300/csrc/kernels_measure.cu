@@ -17,6 +17,7 @@
 #include <cstring>
 
 #include "device.cuh"
+#include "float_sum.cuh"
 #include "internal.h"
 #include "prof.h"
 
@@ -100,11 +101,13 @@ __global__ void __launch_bounds__(256) marginal_partial_kernel(const V<R> *__res
 // thread holds 16 amplitudes that differ in the lowest 4 of those (16 loads in
 // flight), its low 8 index bits are its own, and the block walks the other free
 // bits with the group's high bits fixed: one outcome per thread until the high
-// outcome changes, one register sum (runs of 64 in the state's precision, then
-// FP64), and a shuffle over the lanes that share an outcome before the
-// histogram. Bound by memory: n = 27 complex64, 8 qubits of which 3 are lane
-// bits and the lowest above them is bit 11: 0.17 ms, 0.36 with a histogram add
-// per run of 2^11 amplitudes.
+// outcome changes, one FP64 sum, and a shuffle over the lanes that share an
+// outcome before the histogram. FP64 takes the sums of 2^LV products (in pairs,
+// fours, ...): 16, or as many as the runs of marginal_partial_kernel hold where
+// the group's lowest bit above 8 leaves them shorter (bit 8: every product).
+// Bound by memory: n = 27 complex64, 8 qubits of which 3 are lane bits and the
+// lowest above them is bit 11: 0.17 ms, 0.36 with a histogram add per run of
+// 2^11 amplitudes.
 struct MargWalkP {
     int pos[kMarginalMaxQubits];
     int m;
@@ -114,10 +117,11 @@ struct MargWalkP {
     uint64_t high;      // the group's bits above 8
     int nrest;          // bits of rest
     uint32_t lanes;     // lane bits the group has
+    int lv;             // products summed in the state's precision: 2^lv
     uint64_t chunks;    // per member: 2^(n - 12)
 };
 
-template <typename R>
+template <typename R, int LV>
 __global__ void __launch_bounds__(256) marginal_walk_kernel(const V<R> *__restrict__ psi, const MargWalkP p,
                                                             double *__restrict__ part) {
     __shared__ double h[1 << kMarginalMaxQubits];
@@ -137,26 +141,44 @@ __global__ void __launch_bounds__(256) marginal_walk_kernel(const V<R> *__restri
     uint64_t off[4];
 #pragma unroll
     for (int j = 0; j < 4; ++j) off[j] = 1ull << p.reg[j];
+    // more than 2 FP64 sums per chunk go through FloatSum
+    constexpr bool kFloats = sizeof(R) == 4 && LV <= 2;
     double acc = 0.0;
-    R run = 0;
-    int runs = 0;
-    for (uint64_t k = k0; k < k1; ++k) {
-        const V<R> *b = q + (xr | xh);
-        V<R> a[16];
+    FloatSum fs;
+    for (uint64_t k = k0; k < k1;) {
+        bool done;  // the high outcome ends here, or the block's range
+#pragma unroll 1
+        for (int i = 0; i < 8; ++i) {
+            const V<R> *b = q + (xr | xh);
+            V<R> a[16];
 #pragma unroll
-        for (int c = 0; c < 16; ++c)
-            a[c] = b[((c & 1) ? off[0] : 0ull) | ((c & 2) ? off[1] : 0ull) | ((c & 4) ? off[2] : 0ull) |
-                     ((c & 8) ? off[3] : 0ull)];
+            for (int c = 0; c < 16; ++c)
+                a[c] = b[((c & 1) ? off[0] : 0ull) | ((c & 2) ? off[1] : 0ull) | ((c & 4) ? off[2] : 0ull) |
+                         ((c & 8) ? off[3] : 0ull)];
+            R pr[16];
 #pragma unroll
-        for (int c = 0; c < 16; ++c) run += a[c].x * a[c].x + a[c].y * a[c].y;
-        xr = (xr - p.rest) & p.rest;
-        const bool flush = xr == 0 || k + 1 == k1;
-        if (++runs == 4 || flush) {
-            acc += (double)run;
-            run = 0;
-            runs = 0;
+            for (int c = 0; c < 16; ++c) pr[c] = a[c].x * a[c].x + a[c].y * a[c].y;
+#pragma unroll
+            for (int l = 0; l < LV; ++l)
+#pragma unroll
+                for (int j = 0; j < (16 >> (l + 1)); ++j) pr[j] = pr[2 * j] + pr[2 * j + 1];
+            if constexpr (kFloats) {
+#pragma unroll
+                for (int j = 0; j < (16 >> LV); j += 4) fs.add(pr + j);
+            } else {
+#pragma unroll
+                for (int j = 0; j < (16 >> LV); ++j) acc += (double)pr[j];
+            }
+            xr = (xr - p.rest) & p.rest;
+            done = ++k == k1 || xr == 0;
+            if (done) break;
         }
-        if (flush) {
+        if constexpr (kFloats) {
+            fs.flush();
+            acc += fs.sum;
+            fs.sum = 0.0;
+        }
+        if (done) {
             const uint64_t x = xh | threadIdx.x;
             uint32_t y = 0;
             for (int j = 0; j < p.m; ++j) y |= (uint32_t)((x >> p.pos[j]) & 1ull) << (p.m - 1 - j);
@@ -208,6 +230,7 @@ static bool marginal_walk(const qs_state *s, const MargP &p, MargWalkP *w) {
         else if (regs < 4) w->reg[regs++] = b;
         else w->rest |= 1ull << b, ++w->nrest;
     }
+    w->lv = w->high ? std::min(4, __builtin_ctzll(w->high) - 8) : 4;
     w->chunks = s->n >= 12 ? 1ull << (s->n - 12) : 0;
     return regs == 4;
 }
@@ -235,10 +258,19 @@ qs_status k_marginal(qs_state *s, const int *bitpos, int m, double *out_dev) {
     const dim3 grid((unsigned)parts, (unsigned)s->batch);
     MargWalkP w;
     if (marginal_walk(s, p, &w)) {
-        if (s->dtype == QS_C64)
-            marginal_walk_kernel<float><<<grid, 256, 0, s->stream>>>((const float2 *)s->data, w, part);
+        const float2 *f = (const float2 *)s->data;
+        if (s->dtype == QS_C128)
+            marginal_walk_kernel<double, 4><<<grid, 256, 0, s->stream>>>((const double2 *)s->data, w, part);
+        else if (w.lv == 4)
+            marginal_walk_kernel<float, 4><<<grid, 256, 0, s->stream>>>(f, w, part);
+        else if (w.lv == 3)
+            marginal_walk_kernel<float, 3><<<grid, 256, 0, s->stream>>>(f, w, part);
+        else if (w.lv == 2)
+            marginal_walk_kernel<float, 2><<<grid, 256, 0, s->stream>>>(f, w, part);
+        else if (w.lv == 1)
+            marginal_walk_kernel<float, 1><<<grid, 256, 0, s->stream>>>(f, w, part);
         else
-            marginal_walk_kernel<double><<<grid, 256, 0, s->stream>>>((const double2 *)s->data, w, part);
+            marginal_walk_kernel<float, 0><<<grid, 256, 0, s->stream>>>(f, w, part);
     } else if (s->dtype == QS_C64) {
         marginal_partial_kernel<float><<<grid, 256, 0, s->stream>>>((const float2 *)s->data, p, part);
     } else {

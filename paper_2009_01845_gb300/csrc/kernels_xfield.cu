@@ -17,16 +17,17 @@
 //
 // Per thread the 16 products of a term are summed in the state's precision (8
 // at a time) and added to a running sum that keeps what FP64 would: complex64
-// sums the terms of 8 tiles exactly, as three floats (Knuth's two-sum twice),
-// and adds those to an FP64 sum; an FP64 addition per term would take as long
-// as the read of the state (2 per clock and SM), and a pair of floats (0.56 ms
-// at n = 27) holds 48 bits where FP64 holds 53. FP64 across threads. A state of
-// one tile (n = 12) has its complex64 products added in FP64 one by one, as
-// expect_partial_kernel does there: 26 us, 14 us in lumps of 16 products.
+// sums the terms of 8 tiles exactly, as three floats, and adds those to an FP64
+// sum (float_sum.cuh); an FP64 addition per term would take as long as the read
+// of the state, and a pair of floats (0.56 ms at n = 27) holds 48 bits where FP64
+// holds 53. FP64 across threads. A state of one tile (n = 12) has its complex64
+// products added in FP64 one by one, as expect_partial_kernel does there: 26 us,
+// 14 us in lumps of 16 products.
 #include <algorithm>
 #include <cstring>
 
 #include "device.cuh"
+#include "float_sum.cuh"
 #include "internal.h"
 #include "prof.h"
 #include "xfield.h"
@@ -55,39 +56,7 @@ template <typename R> struct RunningSum {
     __device__ __forceinline__ void flush() {}
     __device__ __forceinline__ double value() const { return (double)s; }
 };
-template <> struct RunningSum<float> {
-    double sum = 0.0;
-    float2 a = {0.f, 0.f}, b = {0.f, 0.f}, c = {0.f, 0.f};  // a + b + c, both lanes: the terms since the last flush
-    __device__ __forceinline__ static float2 two_sum(float2 &s, float2 v) {
-        const float2 t = padd(s, v), bv = psub(t, s);
-        const float2 e = padd(psub(s, psub(t, bv)), psub(v, bv));
-        s = t;
-        return e;
-    }
-    // the four terms of a view (0 where there is none)
-    __device__ __forceinline__ void add(const float *v) {
-        float2 na = a, nb = b, nc = c;
-#pragma unroll
-        for (int j = 0; j < 4; j += 2) {
-            const float2 e = two_sum(na, make_float2(v[j], v[j + 1]));
-            nc = padd(nc, two_sum(nb, e));
-        }
-        if (fabsf(na.x) + fabsf(na.y) <= 3.402823466e38f) {
-            a = na;
-            b = nb;
-            c = nc;
-        } else {  // near the end of the floats' range, infinite or NaN: FP64's result
-            flush();
-            for (int j = 0; j < 4; ++j) sum += (double)v[j];
-        }
-    }
-    __device__ __forceinline__ void flush() {
-        sum += (double)a.x + ((double)b.x + (double)c.x);
-        sum += (double)a.y + ((double)b.y + (double)c.y);
-        a = b = c = make_float2(0.f, 0.f);
-    }
-    __device__ __forceinline__ double value() const { return sum; }
-};
+template <> struct RunningSum<float> : FloatSum {};
 
 // the terms on the 4 register bits of a[], which are tile bits b0 .. b0+3
 template <typename R, bool WIDE>
