@@ -105,9 +105,9 @@ __global__ void __launch_bounds__(256) marginal_partial_kernel(const V<R> *__res
 // outcome before the histogram. FP64 takes the sums of 2^LV products (in pairs,
 // fours, ...): 16, or as many as the runs of marginal_partial_kernel hold where
 // the group's lowest bit above 8 leaves them shorter (bit 8: every product).
-// Bound by memory: n = 27 complex64, 8 qubits of which 3 are lane bits and the
-// lowest above them is bit 11: 0.17 ms, 0.36 with a histogram add per run of
-// 2^11 amplitudes.
+// Bound by memory, with a thread's 16 loads in flight together: 4 CTAs per SM
+// have the 60 registers a thread that takes; left to itself the compiler kept to
+// 40 and issued the loads in parts (n = 32 complex64: 5.9 ms, so 4.9).
 struct MargWalkP {
     int pos[kMarginalMaxQubits];
     int m;
@@ -122,7 +122,7 @@ struct MargWalkP {
 };
 
 template <typename R, int LV>
-__global__ void __launch_bounds__(256) marginal_walk_kernel(const V<R> *__restrict__ psi, const MargWalkP p,
+__global__ void __launch_bounds__(256, 4) marginal_walk_kernel(const V<R> *__restrict__ psi, const MargWalkP p,
                                                             double *__restrict__ part) {
     __shared__ double h[1 << kMarginalMaxQubits];
     const int bins = 1 << p.m;
@@ -213,7 +213,13 @@ __global__ void __launch_bounds__(256) marginal_finalize_kernel(const double *__
     }
 }
 
-// whether the walk takes the group (its 4 register bits exist), and its parameters
+// Whether the walk takes the group (its 4 register bits exist), and its
+// parameters. It is the faster one wherever it applies. Microseconds, complex64,
+// against marginal_partial_kernel, whose runs are short where the group has a low
+// bit above 8: n = 27, one qubit at bit 11 / 16 / 23: 184 / 184 / 184 against
+// 3825 / 267 / 245, 8 lane and warp bits 183 against 207; n = 32, bit 16 / 23:
+// 4964 / 4942 against 5810 / 5604, 12 qubits from the top 4984 against 5617; n =
+// 25, 8 lane and warp bits: 67 against 73. Below n = 19 both take 16 to 20.
 static bool marginal_walk(const qs_state *s, const MargP &p, MargWalkP *w) {
     std::memset(w, 0, sizeof(*w));
     uint64_t group = 0;
