@@ -15,6 +15,7 @@
 
 #include "device.cuh"
 #include "internal.h"
+#include "ising_table.h"
 #include "prof.h"
 #include "tile_device.cuh"
 #include "tiled.h"
@@ -24,15 +25,16 @@ namespace qsim {
 template <typename R> qs_status tile_jit_launch_t(qs_state *s, const TileParams<R> &p, bool *launched);
 
 // The Ising op's tables (see ising_thr_stride), per member (blockIdx.y), in
-// FP64, one thread per entry in the table's own order: for every thread pattern
-// (lane bits, then warp bits) its coupling energy with the fields it puts on the
-// register bits, then each of those fields; the register-pair energies; for
-// every tile the fields of the outside bits on the tile bits and the outside
-// energy. Every energy x is stored as exp(-i tau x). Bound by the FP64 pipe (2
-// operations per clock and SM), so the entries are spread over as many SMs as
-// there are: 64 threads a CTA. A thread per pattern or per tile, 256 a CTA (all
-// patterns of a member on one SM), took 30 us at n = 16 .. 22; 20 steps of two
-// 24-qubit instances, complex64: 6.74 -> 6.16 ms.
+// FP64, one thread per entry (ising_table.h): for every thread pattern (lane
+// bits, then warp bits) its coupling energy with the fields it puts on the
+// register bits, and each of those fields; the register-pair energies; for every
+// tile the fields of the outside bits on the tile bits and the outside energy.
+// Every energy x is stored as exp(-i tau x). Bound by the FP64 pipe (2 operations
+// per clock and SM), so the entries are spread over as many SMs as there are (64
+// threads a CTA) and a warp holds entries of one cost. Per step, 8 instances of
+// 26 qubits, complex64: 100 us (99 with a thread per tile and per pattern, 385
+// with the entries in the table's own order, each outside energy between the
+// tile's fields); one of 26, 25 us (65 and 55); 16 of 16 qubits, 19 us (23 and 20).
 constexpr int kIsingTabThreads = 64;
 
 __global__ void __launch_bounds__(kIsingTabThreads) ising_table_kernel(const __grid_constant__ IsingTabP tp) {
@@ -40,57 +42,58 @@ __global__ void __launch_bounds__(kIsingTabThreads) ising_table_kernel(const __g
     const double *J = tp.ising + (size_t)member * tp.ising_stride;
     const double *hv = J + (size_t)nq * nq;
     double2 *base = reinterpret_cast<double2 *>(tp.out + (size_t)member * tp.stride);
-    const uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const uint64_t patterns = (uint64_t)(1 + tp.rb) << tp.tb, pairs = patterns + (1u << tp.rb);
-    if (i >= pairs + ((uint64_t)(tp.k + 1) << tp.n_free)) return;
-    double x;
-    if (i < patterns) {
-        const int tid = (int)(i / (1 + tp.rb)), c = (int)(i % (1 + tp.rb));
-        auto z = [&](int b) { return ((tid >> b) & 1) ? -1.0 : 1.0; };
-        auto field = [&](int j) {  // on register bit j
-            double w = 0.0;
-            for (int b = 0; b < tp.tb; ++b) w += J[tp.rg[j] * nq + tp.tg[b]] * z(b);
-            return w;
-        };
-        if (c > 0) {
-            x = -2.0 * field(c - 1);
-        } else {
-            double e = 0.0, wsum = 0.0;
-            for (int a = 0; a < tp.tb; ++a)
-                for (int b = a + 1; b < tp.tb; ++b) e += J[tp.tg[a] * nq + tp.tg[b]] * z(a) * z(b);
-            for (int j = 0; j < tp.rb; ++j) wsum += field(j);
-            x = e + wsum;
-        }
-    } else if (i < pairs) {
-        const int r = (int)(i - patterns);
-        x = 0.0;
+    const IsingEntry e =
+        ising_entry((uint64_t)blockIdx.x * blockDim.x + threadIdx.x, tp.tb, tp.rb, tp.k, tp.n_free);
+    const uint32_t row = e.row;
+    auto z = [&](int b) { return ((row >> b) & 1u) ? -1.0 : 1.0; };
+    auto pattern_field = [&](int j) {  // on register bit j
+        double w = 0.0;
+        for (int b = 0; b < tp.tb; ++b) w += J[tp.rg[j] * nq + tp.tg[b]] * z(b);
+        return w;
+    };
+    // h and the couplings of bit g with the outside bits from `from` on (bit o of
+    // a tile's number is the outside bit og[o])
+    auto tile_field = [&](int g, int from) {
+        double acc = hv[g];
+        for (int o = from; o < tp.n_free; ++o) acc += ((row >> o) & 1u) ? -J[g * nq + tp.og[o]] : J[g * nq + tp.og[o]];
+        return acc;
+    };
+    double x = 0.0;
+    switch (e.kind) {
+    case ISING_TILE_FIELD:
+        x = tile_field(tp.gb[e.col], 0);
+        break;
+    case ISING_PATTERN_FIELD:
+        x = -2.0 * pattern_field(e.col);
+        break;
+    case ISING_PAIRS:
         for (int a = 0; a < tp.rb; ++a)
             for (int b = a + 1; b < tp.rb; ++b) {
                 const double c = J[tp.rg[a] * nq + tp.rg[b]];
-                x += (((r >> a) ^ (r >> b)) & 1) ? -c : c;
+                x += (((row >> a) ^ (row >> b)) & 1u) ? -c : c;
             }
-    } else {
-        // bit o of a tile's number is the outside bit og[o]
-        const uint64_t t = (i - pairs) / (tp.k + 1);
-        const int c = (int)((i - pairs) % (tp.k + 1));
-        auto sum = [&](int g, int from) {  // h and the couplings of bit g with the outside bits from `from` on
-            double acc = hv[g];
-            for (int o = from; o < tp.n_free; ++o) acc += ((t >> o) & 1ull) ? -J[g * nq + tp.og[o]] : J[g * nq + tp.og[o]];
-            return acc;
-        };
-        if (c < tp.k) {
-            x = sum(tp.gb[c], 0);
-        } else {
-            x = hv[nq];
-            for (int o = 0; o < tp.n_free; ++o) x += (((t >> o) & 1ull) ? -1.0 : 1.0) * sum(tp.og[o], o + 1);
-        }
+        break;
+    case ISING_TILE_ENERGY:
+        x = hv[nq];
+        for (int o = 0; o < tp.n_free; ++o) x += (((row >> o) & 1u) ? -1.0 : 1.0) * tile_field(tp.og[o], o + 1);
+        break;
+    case ISING_PATTERN_ENERGY: {
+        double wsum = 0.0;
+        for (int a = 0; a < tp.tb; ++a)
+            for (int b = a + 1; b < tp.tb; ++b) x += J[tp.tg[a] * nq + tp.tg[b]] * z(a) * z(b);
+        for (int j = 0; j < tp.rb; ++j) wsum += pattern_field(j);
+        x += wsum;
+        break;
+    }
+    default:
+        return;
     }
     if (tp.single) {
         const V<float> v = expi<float>(-tp.tau * x);
-        base[i] = make_double2(v.x, v.y);
+        base[e.at] = make_double2(v.x, v.y);
     } else {
         const V<double> v = expi<double>(-tp.tau * x);
-        base[i] = make_double2(v.x, v.y);
+        base[e.at] = make_double2(v.x, v.y);
     }
 }
 
@@ -103,8 +106,8 @@ qs_status k_ising_table(qs_state *s, const IsingTabP &in) {
     int no = 0;
     for (int b = 0; b < tp.nq; ++b)
         if (!((tile >> b) & 1ull)) tp.og[no++] = (int8_t)b;
-    const uint64_t entries = ((uint64_t)(1 + tp.rb) << tp.tb) + (1u << tp.rb) + ((uint64_t)(tp.k + 1) << tp.n_free);
-    const dim3 grid((unsigned)((entries + kIsingTabThreads - 1) / kIsingTabThreads), (unsigned)tp.members);
+    const uint64_t threads = ising_threads(tp.tb, tp.rb, tp.k, tp.n_free);
+    const dim3 grid((unsigned)((threads + kIsingTabThreads - 1) / kIsingTabThreads), (unsigned)tp.members);
     ising_table_kernel<<<grid, kIsingTabThreads, 0, s->stream>>>(tp);
     QS_CUDA_TRY(cudaGetLastError());
     return QS_OK;
