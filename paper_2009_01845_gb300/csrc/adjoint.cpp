@@ -114,8 +114,8 @@ qs_status energy_gradient(qs_state *w, const std::vector<LGate> &G, const double
         if (init_zero) QS_TRY(k_init_basis(phi, 0));
         for (int c = 0; c < nseg; ++c) {
             std::vector<LGate> part(G.begin() + (size_t)c * seg, G.begin() + std::min<size_t>(N, (size_t)(c + 1) * seg));
-            QS_TRY(small_state(phi) ? run_small(phi, part, params, n_params)
-                                    : run_tiled(phi, part, params, n_params));
+            QS_TRY(one_launch(phi, part) ? run_small(phi, part, params, n_params)
+                                         : run_tiled(phi, part, params, n_params));
             if (c + 1 < nseg) QS_TRY(copy_phi(w, ckpt[c], true));
         }
         return QS_OK;

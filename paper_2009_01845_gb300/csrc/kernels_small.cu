@@ -476,6 +476,42 @@ qs_status run_t(qs_state *s, const std::vector<LGate> &G, const double *params, 
 
 bool small_state(const qs_state *s) { return s->n < tile_bits(s->dtype); }
 
+// Where the one launch is the faster form. It costs 8 us more than a first gate's
+// launch (descriptors, the state's copy in shared memory) and saves 3.5 us for
+// every further gate while launches bound both; a large batch fills the chip in
+// one-gate launches too, and CTAs that hold a member each then only add the
+// copies and the descriptors, so the batch it may have grows with the gates.
+// Time against a launch per gate, mean of queues of mixed, dense 1-qubit, CZ and
+// dense 2-qubit gates (65535 members: 30 gates and more):
+//   complex64   n =  4: 3 gates 1.0, 4 gates 0.91; 30 gates at 64 / 8192 / 65535
+//               members 0.42 / 0.59 / 1.6; n = 8: 0.41 / 0.92 / 1.2; n = 10, at 64 /
+//               2048 / 65535: 0.42 / 0.99 / 1.3; n = 12: 0.49 / 0.93 / 0.73
+//   complex128  n =  4: 0.47 / 1.04 / 3.0; n = 8, at 64 / 2048 / 65535: 0.46 / 0.84 / 1.3;
+//               n = 11, at 64 / 256 / 65535: 0.64 / 0.80 / 1.4
+// Per-member angles cost one-gate launches a sine and cosine per pair of
+// amplitudes, here one per member: complex128 from n = 6 on 0.26 to 0.91 at any
+// batch, complex64 at n = 12 0.28 to 0.80; at n = 10 with 76 gates 0.29 (256
+// members), 1.04 (4096), 1.4 (65535).
+bool one_launch(const qs_state *s, const std::vector<LGate> &G) {
+    if (!small_state(s)) return false;
+    const bool c64 = s->dtype == QS_C64;
+    const int n = s->n, gates = (int)std::min<size_t>(G.size(), 1u << 20);
+    int angles = 0;
+    for (const LGate &g : G) angles += g.param_index >= 0;
+    int members;  // per gate
+    if (angles > 0 && 4ll * angles >= gates) {
+        if (gates < 3) return false;
+        if (n >= (c64 ? 11 : 6)) return true;
+        members = 1 << std::min(10, 17 - n);
+    } else {
+        if (gates < 4) return false;
+        if (c64 && n == 12 && gates >= 16) return true;
+        members = c64 ? std::min(1 << 9, std::max(1 << 6, (1 << 16) >> n))
+                      : std::min(1 << 7, std::max(1 << 4, (1 << 14) >> n));
+    }
+    return s->batch <= members * std::min(gates, 32);
+}
+
 qs_status run_small(qs_state *s, const std::vector<LGate> &G, const double *params, int n_params, double param_sign,
                     double *gpart) {
     return s->dtype == QS_C64 ? run_t<float>(s, G, params, n_params, param_sign, gpart)

@@ -38,7 +38,7 @@ qs_status run_gates(qs_state *s, std::vector<LGate> &gates, int mode, const qs_o
     case QS_MODE_AUTO:
     case QS_MODE_TILED:
     default:
-        if (small_state(s)) return run_small(s, gates, params_dev, n_params);
+        if (one_launch(s, gates)) return run_small(s, gates, params_dev, n_params);
         return run_tiled(s, gates, params_dev, n_params);
     }
 }
@@ -105,7 +105,7 @@ static qs_status x_layer(qs_state *s, const TrotterTerms &tt, double sv, double 
         QS_TRY(lower_gate(n, g, &lg));
         layer.push_back(std::move(lg));
     }
-    if (small_state(s)) return run_small(s, layer, nullptr, 0);
+    if (one_launch(s, layer)) return run_small(s, layer, nullptr, 0);
     for (const LGate &lg : layer) QS_TRY(k_apply_unfused(s, lg));
     return QS_OK;
 }

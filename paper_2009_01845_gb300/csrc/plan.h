@@ -29,7 +29,7 @@ TileSchedule tile_schedule();  // the calling thread's (default: {0, 0})
 void set_tile_schedule(TileSchedule s);
 
 // Tiled multi-gate passes (one pass per gate for gates a tile cannot express
-// and for states smaller than a tile, which run_gates gives to run_small).
+// and for states smaller than a tile: those that one_launch leaves here).
 // force_bit >= 0 (adjoint sweep): that index bit is kept in every tile and
 // every stage's register set (it is the top register bit); gradient ops write
 // per-tile partials to gpart; batched-parameter gates use angle * param_sign.

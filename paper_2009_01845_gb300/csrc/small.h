@@ -10,6 +10,9 @@ namespace qsim {
 // Whether a state of n qubits is one the small-state kernel holds (the widths
 // the tiled passes do not take).
 bool small_state(const qs_state *s);
+// Whether the kernel takes the queue in place of a launch per gate: the state is
+// one it holds, and gates and members are ones it is the faster form for.
+bool one_launch(const qs_state *s, const std::vector<LGate> &G);
 
 // Apply the queue to every member, in as few launches as its descriptors need.
 // Batched-parameter gates take angle * param_sign; gradient ops (kind
