@@ -74,8 +74,9 @@ uint64_t target_bits(const LGate &g, GClass c) {
 // the high (non-lane) ones: the tile has to include them
 uint64_t need_bits(const LGate &g, GClass c) { return target_bits(g, c) & ~((1ull << kTileLaneBits) - 1ull); }
 
-// 2-qubit gates of lane bits in one pass: a specialised pass with 16 of them
-// takes 5.5 s to compile, and the time grows faster than their number
+// 2-qubit gates with a target among the lane bits in one pass: a specialised
+// pass with 16 of them takes 5.5 s to compile, and the time grows faster than
+// their number (controls on lane bits only select threads)
 constexpr int kMaxLowPairs = 16;
 
 int mat_entries(GClass c) {
@@ -1457,7 +1458,8 @@ qs_status run_tiled(qs_state *s, const std::vector<LGate> &G, const double *para
                     blocked |= qb;
                     continue;
                 }
-                if (cls[i] == G_DENSE2 && (qb & ((1ull << kTileLaneBits) - 1ull)) && ++low2 > kMaxLowPairs) {
+                const uint64_t low = target_bits(G[i], cls[i]) & ((1ull << kTileLaneBits) - 1ull);
+                if (cls[i] == G_DENSE2 && low != 0 && ++low2 > kMaxLowPairs) {
                     blocked |= qb;
                     continue;
                 }

@@ -1,0 +1,31 @@
+"""The planner's cap on 2-qubit gates of the low index bits (CPU, emulated
+passes): 20 of them take two passes, 20 whose low bit is only a control take one."""
+import ctypes
+
+import numpy as np
+import pytest
+
+import oracle
+from paper_2009_01845_gb300 import inputs as qi
+from paper_2009_01845_gb300 import qsim
+from test_planner_emulated import TOL, emu  # noqa: F401 (fixture)
+
+
+@pytest.mark.parametrize("dtype,low_target,passes", [(0, False, 1), (1, False, 1), (0, True, 2)])
+def test_cap_counts_targets(emu, dtype, low_target, passes):  # noqa: F811
+    n, r = 13, qi.rng(3)
+    q = lambda bit: n - 1 - bit  # noqa: E731
+    gates = []
+    for k in range(20):
+        if low_target:
+            gates.append(qi.Gate("UNITARY", (q(7), q(k % 5)), (), (), qi.random_unitary(2, r)))
+        else:
+            gates.append(qi.Gate("UNITARY", (q(7), q(8)), (q(k % 5),), (), qi.random_unitary(2, r)))
+    psi0 = qi.random_state(n, 1)
+    psi = np.array(psi0, dtype=np.complex128)
+    arr, keep = qsim.marshal_gates(gates)
+    count = ctypes.c_int()
+    assert emu.emu_apply_schedule(n, dtype, arr, len(gates), psi.ctypes.data, 0, 0, ctypes.byref(count)) == 0
+    del keep
+    assert np.max(np.abs(psi - oracle.run_circuit(n, gates, psi0))) < TOL[dtype]
+    assert count.value == passes
