@@ -297,6 +297,10 @@ constexpr int kScanChunk = 1024;    // block sums per CTA of the first scan leve
 constexpr int kSegs = 32;           // points of a block whose cumulative sums are kept (every 128 amplitudes)
 constexpr int kGroups = kSampleBlock / 32;  // warp-wide groups of a block
 
+// |a|^2 of the sampling kernels, rounded in one way: the walk must find the sums
+// that block_sums_kernel formed for it
+template <typename R> __device__ __forceinline__ R prob(V<R> a) { return fma(a.x, a.x, a.y * a.y); }
+
 // sum of |psi|^2 over each block of L amplitudes (one CTA of 256 threads per
 // block): per-thread sums in the state's precision, the block total in FP64.
 // WHOLE (L = kSampleBlock): all 16 loads of a thread in flight, and the sum of
@@ -318,7 +322,7 @@ __global__ void __launch_bounds__(256) block_sums_kernel(const V<R> *__restrict_
         for (int j = 0; j < N; ++j) a[j] = b[threadIdx.x + 256 * j];
         R pr[N];
 #pragma unroll
-        for (int j = 0; j < N; ++j) pr[j] = a[j].x * a[j].x + a[j].y * a[j].y;
+        for (int j = 0; j < N; ++j) pr[j] = prob<R>(a[j]);
 #pragma unroll
         for (int j = 0; j < N; ++j) acc += pr[j];
         // level l: lanes that differ in bit l add up half of the groups each
@@ -338,8 +342,7 @@ __global__ void __launch_bounds__(256) block_sums_kernel(const V<R> *__restrict_
         if (lane < 16) gsum[(uint64_t)blockIdx.x * kGroups + j * 8 + (threadIdx.x >> 5)] = pr[0];
     } else {
         for (uint64_t i = threadIdx.x; i < L; i += blockDim.x) {
-            const V<R> a = b[i];
-            acc += a.x * a.x + a.y * a.y;
+            acc += prob<R>(b[i]);
         }
     }
     double d = (double)acc;
@@ -431,8 +434,8 @@ __global__ void __launch_bounds__(kScanChunk) add_offsets_kernel(double *__restr
 // one warp per shot: the smallest x with cdf(x) > u * total. With seg, the walk
 // starts at the block's first segment of 128 amplitudes that can hold it: 32
 // points and a few groups are read instead of up to 4096 amplitudes (10^5 shots
-// at n = 27 complex64: 2.2 ms without). Sums are the same either way: the points
-// are the walk's own running sums, and a segment is passed over only if the
+// at n = 27 complex64: 2.2 ms without). Samples are the same either way: the points
+// are the walk's own running sums (prob() and the order of a warp's scan in both), and a segment is passed over only if the
 // walk could not have stopped in it (a group's scan exceeds its sum by 5
 // roundings at most: 2^-17 of the segment is allowed here, and 2 roundings of
 // the running sum).
@@ -478,10 +481,7 @@ __global__ void __launch_bounds__(256) sample_kernel(const V<R> *__restrict__ q,
     for (int pass = 0; pass < 2; ++pass) {
         for (uint64_t c = start; c < L; c += 32) {
             R pr = 0;
-            if (c + lane < L) {
-                const V<R> a = b[c + lane];
-                pr = a.x * a.x + a.y * a.y;
-            }
+            if (c + lane < L) pr = prob<R>(b[c + lane]);
             R sc = pr;  // inclusive warp scan
 #pragma unroll
             for (int o = 1; o < 32; o <<= 1) {
