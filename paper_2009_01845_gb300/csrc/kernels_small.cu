@@ -6,10 +6,12 @@
 // batch member loads the member into shared memory, applies the queue's gates
 // one after the other (a barrier between gates, none between diagonal gates,
 // whose amplitudes stay with their threads) and stores it back. Each gate's
-// arithmetic is that of its one-gate kernel (kernels_basic.cu,
-// kernels_dfloat.cu), operation for operation, so results are the same bits;
-// the sines and cosines of per-member angles are formed once per launch, one
-// thread per gate. Descriptors and matrices are kernel parameters (up to 32
+// arithmetic has its one-gate kernel's precision and order of products
+// (kernels_basic.cu, kernels_dfloat.cu); per-member rotations leave out the
+// products with entries that are zero, and the two may fuse different products,
+// so results agree to an FMA's rounding (a few 2^-24 per gate in complex64). The
+// sines and cosines of per-member angles are formed once per launch, one thread
+// per gate. Descriptors and matrices are kernel parameters (up to 32
 // KB a launch: 512 gates), so a captured graph holds them by value; the CTA
 // copies them to shared memory first.
 //
@@ -313,7 +315,7 @@ __global__ void __launch_bounds__(kMaxThreads) small_kernel(V<R> *__restrict__ p
             for (int x = tid; x < size; x += nt) {
                 if ((x & op.mask) != op.mask) continue;
                 int l = 0;
-                                for (int j = 0; j < op.k; ++j) l = (l << 1) | ((x >> ((pos >> (5 * j)) & 31u)) & 1);
+                for (int j = 0; j < op.k; ++j) l = (l << 1) | ((x >> ((pos >> (5 * j)) & 31u)) & 1);
                 s[x] = cmul<R>(s[x], mat[op.m + l]);
             }
             break;

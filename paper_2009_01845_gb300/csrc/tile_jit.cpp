@@ -613,7 +613,10 @@ qs_status tile_jit_launch_t(qs_state *s, const TileParams<R> &p, bool *launched)
     // keys: flags (kTypeCode, kKeyFolded: values compiled in), then the
     // descriptor with its run-time pointers and the Ising op's tau (which only
     // the table kernel reads) cleared; the structure key also clears the
-    // values (matrix entries, diagonal factors) but for signs
+    // values (matrix entries, diagonal factors) but for the +-1 constants of
+    // blocks of signs alone: each pattern of them is a kernel of its own (as
+    // each set of thread-bit factors always was), and a program that draws new
+    // patterns compiles new kernels up to the table's 1024 entries
     static thread_local std::vector<unsigned char> full, key;  // reused between launches
     const std::vector<DiagBlock> blocks = diag_blocks<R>(p);
     const size_t bytes = 1 + sizeof(TileParams<R>);
