@@ -6,12 +6,14 @@
 //     gates need no tile bits at all, since a tile knows every index bit of
 //     every amplitude it holds.
 // A gate the tile cannot express (dense on 3+ qubits, a general 2+-qubit
-// diagonal, in double-float a 2-qubit gate of a lane bit) is applied by its own
-// unfused pass when it reaches the front of the queue. Within a pass, stages re-split
+// diagonal, in complex128 a dense 2-qubit gate of a lane bit and in double-float
+// such a SWAP) is applied by its own unfused pass when it reaches the front of the
+// queue, as are one or two 2-qubit gates of lane bits that nothing else joins. Within a pass, stages re-split
 // the tile's bits, lane bits included, between registers, lanes and warps; the
 // register set of a new stage is the needed bits plus the bits used soonest
 // afterwards (furthest-next-use eviction).
 #include <algorithm>
+#include <cmath>
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
@@ -34,11 +36,14 @@ namespace {
 
 enum GClass { G_PHASE, G_DIAG1, G_DENSE1, G_DENSE2, G_SWAP, G_GRAD, G_ISING, G_SINGLE };
 
-// low_pairs: 2-qubit gates and SWAPs that touch a lane bit may run in a tile too.
-// Complex128 in double-float keeps those in passes of their own: one-gate SWAPs
-// move amplitudes exactly, and a double-float 4x4 gate makes a specialised pass
-// slow to compile (2 of them 14 s, 4 of them 47 s).
-GClass classify(const LGate &g, bool low_pairs) {
+// low_swaps, low_dense: SWAPs and dense 2-qubit gates with a target on a lane
+// bit may run in a tile too. Complex128 in double-float keeps both in passes of
+// their own: one-gate SWAPs move amplitudes exactly, and a double-float 4x4 gate
+// makes a specialised pass slow to compile (2 of them 14 s, 4 of them 47 s). In
+// FP64 the dense ones stay alone as well: the FP64 pipe bounds them either way
+// (n = 26: 2.06 ms alone, 2.01 as one of two in a tile), and a tile does not skip
+// what controls leave out (0.53 ms with 2 controls alone, 1.45 in a tile).
+GClass classify(const LGate &g, bool low_swaps, bool low_dense) {
     if (g.kind == kKindGrad) return G_GRAD;
     if (g.kind == kKindIsing) return G_ISING;
     if (g.param_index >= 0) {
@@ -52,10 +57,10 @@ GClass classify(const LGate &g, bool low_pairs) {
     }
     if (g.phase_only) return G_PHASE;
     if (g.diagonal) return g.k == 1 ? G_DIAG1 : G_SINGLE;
-    const bool pair = g.k == 2 && (low_pairs || (g.tbit[0] >= kTileLaneBits && g.tbit[1] >= kTileLaneBits));
-    if (g.is_swap) return pair ? G_SWAP : G_SINGLE;
     if (g.k == 1) return G_DENSE1;
-    return pair ? G_DENSE2 : G_SINGLE;
+    const bool high = g.k == 2 && g.tbit[0] >= kTileLaneBits && g.tbit[1] >= kTileLaneBits;
+    if (g.is_swap) return high || low_swaps ? G_SWAP : G_SINGLE;
+    return high || (g.k == 2 && low_dense) ? G_DENSE2 : G_SINGLE;
 }
 
 uint64_t qubit_bits(const LGate &g) {
@@ -78,6 +83,25 @@ uint64_t need_bits(const LGate &g, GClass c) { return target_bits(g, c) & ~((1ul
 // pass with 16 of them takes 5.5 s to compile, and the time grows faster than
 // their number (controls on lane bits only select threads)
 constexpr int kMaxLowPairs = 16;
+
+// Whether a pass would hold nothing but low pairs, and so few of them that their
+// own passes are faster: those read only what the controls select, and need no
+// tile. Microseconds of one launch each against the tiled pass (generic and
+// specialised), complex64: n = 27, a dense 2-qubit gate 348 / 518 and 376, with 2
+// controls 98 / 482 and 382, a SWAP 325 / 402 and 390, two dense gates 664 / 637
+// and 394; n = 22, two dense gates 38 / 49 and 42; n = 14, one 20 / 28, two 26 / 39.
+bool only_few_low_pairs(const qs_state *s, const std::vector<LGate> &G, const std::vector<GClass> &cls,
+                        const std::vector<int> &gates) {
+    if (gates.empty()) return false;
+    double reads = 0.0;  // of the state
+    for (int gi : gates) {
+        if (cls[gi] != G_DENSE2 && cls[gi] != G_SWAP) return false;
+        if ((target_bits(G[gi], cls[gi]) & ((1ull << kTileLaneBits) - 1ull)) == 0) return false;
+        reads += std::ldexp(1.0, -__builtin_popcountll(G[gi].cmask));
+    }
+    const uint64_t amplitudes = (uint64_t)s->batch << s->n;
+    return amplitudes <= (1ull << 23) ? gates.size() <= 2 : reads <= 1.0;
+}
 
 int mat_entries(GClass c) {
     switch (c) {
@@ -1411,8 +1435,8 @@ qs_status run_tiled(qs_state *s, const std::vector<LGate> &G, const double *para
     const int nh = k - kTileLaneBits;  // chosen high tile bits
     const uint64_t force = force_bit >= 0 ? (1ull << force_bit) : 0ull;
     std::vector<GClass> cls(G.size());
-    const bool low_pairs = s->dtype == QS_C64 || c128_fp64();
-    for (size_t i = 0; i < G.size(); ++i) cls[i] = classify(G[i], low_pairs);
+    const bool c64 = s->dtype == QS_C64;
+    for (size_t i = 0; i < G.size(); ++i) cls[i] = classify(G[i], c64 || c128_fp64(), c64);
     // per-member matrices of every batched-parameter gate, built once on the device
     std::vector<int> slot(G.size(), -1), spidx, skind;
     for (size_t i = 0; i < G.size(); ++i)
@@ -1482,6 +1506,13 @@ qs_status run_tiled(qs_state *s, const std::vector<LGate> &G, const double *para
                 if (q.gates.size() > pp.gates.size()) pp = std::move(q);
             }
             if (pp.gates.empty() && sched.select == 2) select(false, 0, &pp);
+        }
+        if (only_few_low_pairs(s, G, cls, pp.gates)) {
+            for (int gi : pp.gates) {
+                QS_TRY(k_apply_unfused(s, G[gi]));
+                done[gi] = 1;
+            }
+            continue;
         }
         if (pp.gates.empty()) {
             // the front gate cannot run in a tile

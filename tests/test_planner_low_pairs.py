@@ -29,3 +29,19 @@ def test_cap_counts_targets(emu, dtype, low_target, passes):  # noqa: F811
     del keep
     assert np.max(np.abs(psi - oracle.run_circuit(n, gates, psi0))) < TOL[dtype]
     assert count.value == passes
+
+
+@pytest.mark.parametrize("count,passes", [(1, 0), (2, 0), (3, 1)])
+@pytest.mark.parametrize("kind", ["SWAP", "UNITARY"])
+def test_few_alone_run_one_by_one(emu, kind, count, passes):  # noqa: F811
+    n, r = 14, qi.rng(4)
+    gates = [qi.Gate(kind, (n - 1 - k, 2 * k), (k + 3,) if k % 2 else (),
+                     (), qi.random_unitary(2, r) if kind == "UNITARY" else None) for k in range(count)]
+    psi0 = qi.random_state(n, 2)
+    psi = np.array(psi0, dtype=np.complex128)
+    arr, keep = qsim.marshal_gates(gates)
+    ran = ctypes.c_int()
+    assert emu.emu_apply_schedule(n, 0, arr, len(gates), psi.ctypes.data, 0, 0, ctypes.byref(ran)) == 0
+    del keep
+    assert np.max(np.abs(psi - oracle.run_circuit(n, gates, psi0))) < TOL[0]
+    assert ran.value == passes
