@@ -45,6 +45,7 @@ constexpr int kMaxGroups = 64;  // of each kind, per launch
 constexpr int kMaxTerms = 384;  // of the Z-only and the remaining groups, per launch
 
 template <typename R> struct HpsiP {
+    static constexpr int kOutputs = sizeof(R) == 4 ? 16 : 8;  // per thread, at most
     // constant groups: [0, run_in) and [run_in, run0) share one coefficient
     // (partners inside and outside the tile), then [run0, c_in), [c_in, nc)
     int nc, run_in, run0, c_in;
@@ -65,14 +66,14 @@ template <typename R> struct HpsiP {
     // dmb[m + 1]) are those whose chunk bits are m, without the Ising ones
     int diag;
     uint16_t dord[kMaxTerms];
-    int dmb[9];
+    int dmb[kOutputs + 1];
     // Ising energy qc0 + sum_i qh[i] z_i + sum_{i<j} qJ[i][j] z_i z_j in index
     // bits (z_i = 1 - 2 y_i; qJ symmetric, zero diagonal); qecc: the chunk bits' pairs
     int quad;
     R qc0;
     R qh[32];
     R qJ[32][32];
-    R qecc[8];
+    R qecc[kOutputs];
     int n, ms;
     uint64_t total;
     const void *part;  // partial sums of earlier launches, or null
@@ -384,24 +385,34 @@ __global__ void __launch_bounds__(1 << TB, MINB) hpsi_tile_kernel(const V<R> *__
 // the groups for more outputs at once; small ones give small states enough
 // CTAs (2^16 amplitudes are 256 tiles of 2^8, 16 of 2^12). Microseconds per
 // application (transverse field, dense Ising, 8 strings, Runge-Kutta's two
-// results) with 1, 4, 8 outputs per thread in complex64 and 1, 2, 4 in
-// complex128, at n = 16, 18, 20, 22, 24:
-//   complex64   7.9  13.6  33.5  151  596 | 11.6  12.7  26.6  103  495 | 16.4  16.7  23.0   87   385
-//   complex128 18.5  40.3   135  592 2391 | 22.4  45.6   121  532 2315 | 39.7  41.6   128  482  2059
+// results) with 1, 4, 8 outputs per thread in complex64, at n = 16, 18, 20, 22, 24:
+//   7.9  13.6  33.5  151  596 | 11.6  12.7  26.6  103  495 | 16.4  16.7  23.0   87   385
+// and of a Runge-Kutta step (field, 100 pairs) in complex128 with 1 and 8 outputs:
+//   n = 17  261 317, n = 18  315 327, n = 19  - 354, n = 20  - 543 (2 outputs: 376, 566)
+// (n = 25: 11.7 ms; 4 outputs in 512 threads, 14.4).
+// Z-only strings of weight > 2 (`strings`) are summed per chunk mask, so more
+// outputs per thread share a string's sign; in complex128 each is an FP64 addition.
+// The same step with 250 of them, 1 output (or 2) against 8: n = 16  618 554, n = 17
+// 940 558, n = 18  1556 568, n = 20  2627 1175; with 8 / 32 / 64 of them at n = 18: 352
+// 345, 458 363, 621 391; with 32 / 64 at n = 17: 336 354, 413 386. complex64, 8 outputs
+// of 512 threads against 16 of 256: n = 25, 0 / 80 / 120 / 250 strings, 3.02 3.65, 3.64
+// 3.98, 3.97 4.03, 5.41 4.47 ms (Dormand-Prince 6.70 6.53, 7.20 6.63, 9.49 7.37); n = 19
+// from 4 outputs, 100 / 250 strings, 293 300, 436 392 us.
 struct Shape {
     int tb = 0, pb = 0;
 };
-Shape shape_for(qs_dtype dtype, int n, uint64_t total) {
+Shape shape_for(qs_dtype dtype, int n, uint64_t total, size_t strings) {
     if (n > 32) return {};
     if (dtype == QS_C64) {
+        if (n >= 12 && total >= (1ull << 19) && strings >= 100) return {8, 4};
         if (n >= 12 && total >= (1ull << 20)) return {9, 3};
         if (n >= 10 && total >= (1ull << 18)) return {8, 2};
         return n >= 8 ? Shape{8, 0} : Shape{};
     }
     // below 11 qubits complex128 stays in FP64
     if (n < 11) return {};
-    if (total >= (1ull << 21)) return {9, 2};
-    if (total >= (1ull << 19)) return {8, 1};
+    const uint64_t t = std::min<uint64_t>(total >> 16, 8);
+    if (t == 8 || t * t * strings >= 160) return {8, 3};
     return {8, 0};
 }
 
@@ -609,12 +620,12 @@ qs_status launch_t(const Shape &shape, const V<R> *src, const HpsiP<R> &p, cudaS
         const uint64_t blocks = std::min<uint64_t>((p.total + 255) / 256, (uint64_t)sm_count_hpsi() * 32);
         hpsi_kernel<R><<<(unsigned)std::max<uint64_t>(1, blocks), 256, 0, st>>>(src, p);
     } else if constexpr (sizeof(R) == 4) {
-        if (shape.pb == 3) launch_tile<float, float, 9, 3, 2>(src, p, st);
+        if (shape.pb == 4) launch_tile<float, float, 8, 4, 2>(src, p, st);
+        else if (shape.pb == 3) launch_tile<float, float, 9, 3, 2>(src, p, st);
         else if (shape.pb == 2) launch_tile<float, float, 8, 2, 4>(src, p, st);
         else launch_tile<float, float, 8, 0, 6>(src, p, st);
     } else {
-        if (shape.pb == 2) launch_tile<double, dd, 9, 2, 1>(src, p, st);
-        else if (shape.pb == 1) launch_tile<double, dd, 8, 1, 3>(src, p, st);
+        if (shape.pb == 3) launch_tile<double, dd, 8, 3, 2>(src, p, st);
         else launch_tile<double, dd, 8, 0, 4>(src, p, st);
     }
     QS_CUDA_TRY(cudaGetLastError());
@@ -651,7 +662,9 @@ qs_status hpsi_prepare(const StateView &s, const qs_pauli_term *terms, size_t co
     op->impl = std::make_shared<HpsiOp::Impl>();
     HpsiOp::Impl &im = *op->impl;
     im.shape = s;
-    im.tile = shape_for(s.dtype, s.n, (uint64_t)s.batch << s.n);
+    size_t strings = 0;  // Z-only terms that are not Ising terms
+    for (size_t t = 0; t < count; ++t) strings += terms[t].x_mask == 0 && __builtin_popcountll(terms[t].z_mask) > 2;
+    im.tile = shape_for(s.dtype, s.n, (uint64_t)s.batch << s.n, strings);
     im.terms = (double)count;
     return s.dtype == QS_C64 ? prepare_t<float>(s, im.tile, terms, count, &im.f)
                              : prepare_t<double>(s, im.tile, terms, count, &im.d);
