@@ -565,6 +565,14 @@ qs_status k_sample(qs_state *s, int member, const double *u_dev, uint64_t shots,
         }
     }
     if (!segments) QS_TRY(ensure_scratch(s, base));
+    // In complex128 the groups' sums are FP64 additions (2 per clock and SM) on top
+    // of the blocks': few shots on a large state are faster without them, although
+    // each then walks its block from the start (60 us alone, 0.044 us among many).
+    // 1 / 1000 / 10^4 shots with and without: n = 24  196 199 226 | 247 327 816 us; n =
+    // 26  600 602 630 | 568 577 1080; n = 28  2230 2230 2260 | 1770 1813 2258; n = 30
+    // 8727 8726 8756 | 6714 6735 7211. complex64 has them in FP32 (n = 30, one shot:
+    // 1.44 ms, 2.44 without).
+    if (s->dtype == QS_C128 && nb >= (1u << 14) && shots < nb / 8) segments = false;
     ProfScope _ps(s->stream, KC_REDUCE, (double)per * (s->dtype == QS_C64 ? 8 : 16), 3.0 * per);
     const uint64_t moff = (uint64_t)member << s->ms;
     return s->dtype == QS_C64
