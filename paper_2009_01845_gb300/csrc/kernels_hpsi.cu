@@ -31,6 +31,7 @@
 #include <algorithm>
 #include <cstring>
 #include <type_traits>
+#include <utility>
 #include <vector>
 
 #include "device.cuh"
@@ -178,7 +179,8 @@ template <typename R, typename A, int TB, int PB, int MINB>
 __global__ void __launch_bounds__(1 << TB, MINB) hpsi_tile_kernel(const V<R> *__restrict__ src,
                                                                   const __grid_constant__ HpsiP<R> p) {
     constexpr int T = 1 << TB, PER = 1 << PB, K = TB + PB;
-    constexpr int U = PB >= 3 ? 2 : PB == 2 ? 4 : 8;  // groups whose loads are in flight together
+    // groups whose loads are in flight together (8 double-float partners take 32 registers)
+    constexpr int U = PB >= 3 ? (is_dd<A> ? 1 : 2) : PB == 2 ? 4 : 8;
     __shared__ V<A> tile[1 << K];
     __shared__ R s_w[T];  // transform over the thread bits
     __shared__ R s_f[K];  // Ising fields of the outside bits on the tile bits
@@ -355,7 +357,11 @@ __global__ void __launch_bounds__(1 << TB, MINB) hpsi_tile_kernel(const V<R> *__
                 }
             }
 #pragma unroll
-            for (int j = 0; j < PER; ++j) acc[j] = rmadd<A>(A(D[j]), own[j], acc[j]);
+            for (int j = 0; j < PER; ++j) {
+                // (read back where registers are short)
+                const V<A> v = is_dd<A> && PB >= 3 ? tile[tid + T * j] : own[j];
+                acc[j] = rmadd<A>(A(D[j]), v, acc[j]);
+            }
         }
         // remaining groups
         for (int g = 0; g < p.ng; ++g) {
@@ -387,22 +393,31 @@ __global__ void __launch_bounds__(1 << TB, MINB) hpsi_tile_kernel(const V<R> *__
 // application (transverse field, dense Ising, 8 strings, Runge-Kutta's two
 // results) with 1, 4, 8 outputs per thread in complex64, at n = 16, 18, 20, 22, 24:
 //   7.9  13.6  33.5  151  596 | 11.6  12.7  26.6  103  495 | 16.4  16.7  23.0   87   385
-// and of a Runge-Kutta step (field, 100 pairs) in complex128 with 1 and 8 outputs:
-//   n = 17  261 317, n = 18  315 327, n = 19  - 354, n = 20  - 543 (2 outputs: 376, 566)
-// (n = 25: 11.7 ms; 4 outputs in 512 threads, 14.4).
-// Z-only strings of weight > 2 (`strings`) are summed per chunk mask, so more
-// outputs per thread share a string's sign; in complex128 each is an FP64 addition.
-// The same step with 250 of them, 1 output (or 2) against 8: n = 16  618 554, n = 17
-// 940 558, n = 18  1556 568, n = 20  2627 1175; with 8 / 32 / 64 of them at n = 18: 352
-// 345, 458 363, 621 391; with 32 / 64 at n = 17: 336 354, 413 386. complex64, 8 outputs
-// of 512 threads against 16 of 256: n = 25, 0 / 80 / 120 / 250 strings, 3.02 3.65, 3.64
-// 3.98, 3.97 4.03, 5.41 4.47 ms (Dormand-Prince 6.70 6.53, 7.20 6.63, 9.49 7.37); n = 19
-// from 4 outputs, 100 / 250 strings, 293 300, 436 392 us.
+// and of a Runge-Kutta step in complex128 (field, all pairs, 8 strings) with 1 (n =
+// 18), 2 (20) or 4 (22, 25) outputs against 8: 373 364, 733 687, 2307 1973 us, 18.2 15.0 ms.
+// What moves the lines: Z-only strings of weight > 2 (`strings`) are summed per
+// chunk mask, so more outputs per thread share a string's sign, and in complex128
+// each is an FP64 addition. The same step with 250 of them, 1 output (or 2) against
+// 8: n = 16  618 554, n = 17  940 558, n = 18  1556 568, n = 20  2627 1175; with 8 / 32 /
+// 64 of them at n = 18: 352 345, 458 363, 621 391; with 32 / 64 at n = 17: 336 354, 413
+// 386. Terms with X and Z bits (`mixed`) go the other way in a state of few tiles: n =
+// 17, 40 strings, 0 / 24 / 60 of them, 399 371, 440 490, 530 636. So do X masks with
+// several strings (`several` terms), per output and in FP64: a Heisenberg chain in a
+// field, 2 (n = 19, 20) and 4 outputs against 8: 938 1125, 1735 2181, n = 22  7334 7830,
+// n = 25  63.0 67.0 ms. complex64, 8 outputs of 512 threads against 16 of 256: n = 25,
+// 0 / 80 / 120 / 250 strings, 3.02 3.65, 3.64 3.98, 3.97 4.03, 5.41 4.47 ms (Dormand-Prince
+// 6.70 6.53, 7.20 6.63, 9.49 7.37); n = 19 from 4 outputs, 100 / 250 strings, 293 300,
+// 436 392 us.
 struct Shape {
     int tb = 0, pb = 0;
 };
-Shape shape_for(qs_dtype dtype, int n, uint64_t total, size_t strings) {
+Shape shape_for(qs_dtype dtype, int n, uint64_t total, const qs_pauli_term *terms, size_t count) {
     if (n > 32) return {};
+    size_t strings = 0, mixed = 0;
+    for (size_t t = 0; t < count; ++t) {
+        strings += terms[t].x_mask == 0 && __builtin_popcountll(terms[t].z_mask) > 2;
+        mixed += terms[t].x_mask != 0 && terms[t].z_mask != 0;
+    }
     if (dtype == QS_C64) {
         if (n >= 12 && total >= (1ull << 19) && strings >= 100) return {8, 4};
         if (n >= 12 && total >= (1ull << 20)) return {9, 3};
@@ -411,8 +426,21 @@ Shape shape_for(qs_dtype dtype, int n, uint64_t total, size_t strings) {
     }
     // below 11 qubits complex128 stays in FP64
     if (n < 11) return {};
-    const uint64_t t = std::min<uint64_t>(total >> 16, 8);
-    if (t == 8 || t * t * strings >= 160) return {8, 3};
+    const uint64_t t16 = std::min<uint64_t>(total >> 16, 8);
+    if (t16 == 8 || t16 * t16 * strings >= 160 + 4 * mixed) {
+        std::vector<std::pair<uint64_t, bool>> x;  // X masks, and whether the term has Z bits
+        for (size_t t = 0; t < count && mixed > 0; ++t)
+            if (terms[t].x_mask) x.push_back({terms[t].x_mask, terms[t].z_mask != 0});
+        std::sort(x.begin(), x.end());
+        size_t several = 0;
+        for (size_t i = 0, j; i < x.size(); i = j) {
+            for (j = i; j < x.size() && x[j].first == x[i].first; ++j) {}
+            if (j - i > 1 && x[j - 1].second) several += j - i;
+        }
+        if (several <= strings) return {8, 3};
+    }
+    if (total >= (1ull << 21)) return {9, 2};
+    if (total >= (1ull << 19)) return {8, 1};
     return {8, 0};
 }
 
@@ -626,6 +654,8 @@ qs_status launch_t(const Shape &shape, const V<R> *src, const HpsiP<R> &p, cudaS
         else launch_tile<float, float, 8, 0, 6>(src, p, st);
     } else {
         if (shape.pb == 3) launch_tile<double, dd, 8, 3, 2>(src, p, st);
+        else if (shape.pb == 2) launch_tile<double, dd, 9, 2, 1>(src, p, st);
+        else if (shape.pb == 1) launch_tile<double, dd, 8, 1, 3>(src, p, st);
         else launch_tile<double, dd, 8, 0, 4>(src, p, st);
     }
     QS_CUDA_TRY(cudaGetLastError());
@@ -662,9 +692,7 @@ qs_status hpsi_prepare(const StateView &s, const qs_pauli_term *terms, size_t co
     op->impl = std::make_shared<HpsiOp::Impl>();
     HpsiOp::Impl &im = *op->impl;
     im.shape = s;
-    size_t strings = 0;  // Z-only terms that are not Ising terms
-    for (size_t t = 0; t < count; ++t) strings += terms[t].x_mask == 0 && __builtin_popcountll(terms[t].z_mask) > 2;
-    im.tile = shape_for(s.dtype, s.n, (uint64_t)s.batch << s.n, strings);
+    im.tile = shape_for(s.dtype, s.n, (uint64_t)s.batch << s.n, terms, count);
     im.terms = (double)count;
     return s.dtype == QS_C64 ? prepare_t<float>(s, im.tile, terms, count, &im.f)
                              : prepare_t<double>(s, im.tile, terms, count, &im.d);
