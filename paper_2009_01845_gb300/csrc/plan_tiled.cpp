@@ -8,7 +8,7 @@
 // A gate the tile cannot express (dense on 3+ qubits, a general 2+-qubit
 // diagonal, in complex128 a dense 2-qubit gate of a lane bit and in double-float
 // such a SWAP) is applied by its own unfused pass when it reaches the front of the
-// queue, as are one or two 2-qubit gates of lane bits that nothing else joins. Within a pass, stages re-split
+// queue, as are a few 2-qubit gates of lane bits that nothing else joins. Within a pass, stages re-split
 // the tile's bits, lane bits included, between registers, lanes and warps; the
 // register set of a new stage is the needed bits plus the bits used soonest
 // afterwards (furthest-next-use eviction).
@@ -89,7 +89,9 @@ constexpr int kMaxLowPairs = 16;
 // tile. Microseconds of one launch each against the tiled pass (generic and
 // specialised), complex64: n = 27, a dense 2-qubit gate 348 / 518 and 376, with 2
 // controls 98 / 482 and 382, a SWAP 325 / 402 and 390, two dense gates 664 / 637
-// and 394; n = 22, two dense gates 38 / 49 and 42; n = 14, one 20 / 28, two 26 / 39.
+// and 394; n = 22, two dense gates 38 / 49 and 42, five 76 / 84, four with a
+// control 47 / 73 and 60, eleven SWAPs 112 / 91; n = 13 to 16, one 20 / 28, two 26 /
+// 39, five 42 to 47 / 58 and 52, four with a control 33 to 41 / 50, seven SWAPs 55 / 48.
 bool only_few_low_pairs(const qs_state *s, const std::vector<LGate> &G, const std::vector<GClass> &cls,
                         const std::vector<int> &gates) {
     if (gates.empty()) return false;
@@ -100,7 +102,7 @@ bool only_few_low_pairs(const qs_state *s, const std::vector<LGate> &G, const st
         reads += std::ldexp(1.0, -__builtin_popcountll(G[gi].cmask));
     }
     const uint64_t amplitudes = (uint64_t)s->batch << s->n;
-    return amplitudes <= (1ull << 23) ? gates.size() <= 2 : reads <= 1.0;
+    return amplitudes <= (1ull << 23) ? gates.size() <= 5 : reads <= 1.0;
 }
 
 int mat_entries(GClass c) {

@@ -19,7 +19,7 @@ def queue(name, n):
     return {"dense": [u(q(0), q(3))], "swap": [qi.Gate("SWAP", (q(1), 0))],
             "controlled": [u(q(k), q(9), c=(q(10), q(11))) for k in range(4)],
             "two": [u(q(0), 1), u(q(1), 2)], "beside": [u(q(0), q(3)), qi.Gate("U3", (q(7),), (), (0.1, 0.2, 0.3))],
-            "swaps": [qi.Gate("SWAP", (k, q(k))) for k in range(5)]}[name]
+            "swaps": [qi.Gate("SWAP", (k, q(k))) for k in range(6)]}[name]
 
 
 @pytest.mark.parametrize("dtype,n,name,tiled", [

@@ -1,5 +1,5 @@
 """The planner's cap on 2-qubit gates of the low index bits (CPU, emulated
-passes): 20 of them take two passes, 20 whose low bit is only a control take one."""
+passes): 24 of them take two passes, 24 whose low bit is only a control take one."""
 import ctypes
 
 import numpy as np
@@ -16,7 +16,7 @@ def test_cap_counts_targets(emu, dtype, low_target, passes):  # noqa: F811
     n, r = 13, qi.rng(3)
     q = lambda bit: n - 1 - bit  # noqa: E731
     gates = []
-    for k in range(20):
+    for k in range(24):
         if low_target:
             gates.append(qi.Gate("UNITARY", (q(7), q(k % 5)), (), (), qi.random_unitary(2, r)))
         else:
@@ -31,11 +31,11 @@ def test_cap_counts_targets(emu, dtype, low_target, passes):  # noqa: F811
     assert count.value == passes
 
 
-@pytest.mark.parametrize("count,passes", [(1, 0), (2, 0), (3, 1)])
+@pytest.mark.parametrize("count,passes", [(1, 0), (2, 0), (5, 0), (6, 1)])
 @pytest.mark.parametrize("kind", ["SWAP", "UNITARY"])
 def test_few_alone_run_one_by_one(emu, kind, count, passes):  # noqa: F811
     n, r = 14, qi.rng(4)
-    gates = [qi.Gate(kind, (n - 1 - k, 2 * k), (k + 3,) if k % 2 else (),
+    gates = [qi.Gate(kind, (n - 1 - k % 5, k), (7,) if k % 2 else (),
                      (), qi.random_unitary(2, r) if kind == "UNITARY" else None) for k in range(count)]
     psi0 = qi.random_state(n, 2)
     psi = np.array(psi0, dtype=np.complex128)
